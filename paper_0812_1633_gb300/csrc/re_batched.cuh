@@ -104,9 +104,10 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   BatchedSmem sm;
-  batched_layout(dims.max_n, dims.max_ncell, T, FP64, dims.list_elems, smem_raw, &sm);
-  uint4* posm = reinterpret_cast<uint4*>(sm.pos);
-  Pos64* pos64 = reinterpret_cast<Pos64*>(sm.pos);
+  batched_layout(dims.max_n, T, FP64, dims.list_elems, smem_raw, &sm);
+  // the positions lie at the base of the dynamic shared memory (batched_layout)
+  uint4* posm = reinterpret_cast<uint4*>(smem_raw);
+  Pos64* pos64 = reinterpret_cast<Pos64*>(smem_raw);
 
   // Every CTA has read the replica's flags before any CTA may change them
   // (the barrier also publishes E and K to the whole CTA).
@@ -227,45 +228,17 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
 
   int overflow = 0;
   int nreb = 0;
-  // Rebuild of the lists of this CTA's atoms.  With cells, the lane groups take
-  // this CTA's atoms in cell order (neighbouring lanes then scan the same cell
-  // ranges) and hand the sub-list counts to the owners through shared memory.
+  // Rebuild of the lists of this CTA's atoms.
   auto rebuild = [&]() {
-    if (E.nc > 0) {
-      cta_build_cells(hi_of, N, E.nc, sm.cstart, sm.ccnt, sm.spos, sm.acell, sm.iscr);
-      int n_own = i1 - i0;
-      if (C > 1) {
-        const int pt = (N + T - 1) / T;
-        const int lo = min(N, tid * pt), hi = min(N, lo + pt);
-        int c = 0;
-        for (int k = lo; k < hi; ++k) {
-          const int a = (int)sm.spos[k].w;
-          c += (a >= i0 && a < i1);
-        }
-        sm.wscan[tid] = c;
-        __syncthreads();
-        block_exclusive_scan(sm.wscan, sm.wscan + T + 1, T, sm.iscr);
-        int at = sm.wscan[T + 1 + tid];
-        for (int k = lo; k < hi; ++k) {
-          const int a = (int)sm.spos[k].w;
-          if (a >= i0 && a < i1) sm.own_sorted[at++] = (uint16_t)k;
-        }
-        __syncthreads();
-      }
-      const int gi = tid / P;
-      if (gi < n_own) {
-        // one CTA: every sorted slot is its own; several: the compacted slots
-        const int a = (int)sm.spos[C == 1 ? gi : (int)sm.own_sorted[gi]].w;
-        const uint32_t col = LSM ? (uint32_t)((a - i0) * P + q) : (uint32_t)(a * P + q);
-        const int c = build_sublist<P>(a, q, hi_of, N, E.nc, E.m, sm.cstart, sm.spos, K.rl2u, nb,
-                                       col, ncols, cap_sub, &overflow);
-        sm.cnt_sh[(a - i0) * P + q] = c;
-      }
-      __syncthreads();
-      if (own) cnt = sm.cnt_sh[(i - i0) * P + q];
-    } else if (own) {
-      cnt = build_sublist<P>(i, q, hi_of, N, E.nc, E.m, sm.cstart, sm.spos, K.rl2u, nb, mycol,
-                             ncols, cap_sub, &overflow);
+    if (N <= kDirectBuild * P) {
+      cnt = build_sublist_direct<P>(i, q, own, hi_of, N, K.rl2u, nb, mycol, ncols, cap_sub,
+                                    &overflow);
+    } else {
+      cta_screen_vectors(hi_of, N, sm.hk, sm.box);
+      cnt = build_sublist<P>(i, own, i0 + warp * (32 / P), hi_of, N, sm.hk, sm.box,
+                             sm.act + warp * row_list_bytes(N), K.rl2u, nb, mycol, ncols,
+                             S.raw + rd.nbr_off, (uint32_t)(i * P + q), (uint32_t)(N * P), cap_sub,
+                             &overflow);
     }
     if (own) {
 #pragma unroll
@@ -747,10 +720,10 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
 template <bool FP64, int P, bool LSM, int MODE, int MAXT>
 cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                                    const int* d_work, int n_work, const int32_t* d_budget,
-                                   const LaunchCfg& cfg, int max_n, int max_ncell,
+                                   const LaunchCfg& cfg, int max_n,
                                    size_t list_elems, int async_nx, cudaStream_t st,
                                    const FreeDev* fr) {
-  const size_t smem = batched_smem_bytes(max_n, max_ncell, cfg.threads, FP64, list_elems);
+  const size_t smem = batched_smem_bytes(max_n, cfg.threads, FP64, list_elems);
   auto fn = md_batched_kernel<FP64, P, LSM, MODE, MAXT>;
   cudaFuncAttributes fa{};
   cudaError_t e = cudaFuncGetAttributes(&fa, fn);
@@ -777,7 +750,7 @@ cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDe
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  KernelDims dims{max_n, max_ncell, list_elems, async_nx};
+  KernelDims dims{max_n, list_elems, async_nx};
   FreeDev f{};
   if (fr) f = *fr;
   e = cudaLaunchKernelEx(&lc, fn, s, d_ens, d_rep, d_work, d_budget, dims, f);
@@ -786,9 +759,8 @@ cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDe
 }
 
 template <bool FP64, int P, bool LSM, int MAXT>
-int max_active_clusters_t(const LaunchCfg& cfg, int max_n, int max_ncell,
-                                 size_t list_elems) {
-  const size_t smem = batched_smem_bytes(max_n, max_ncell, cfg.threads, FP64, list_elems);
+int max_active_clusters_t(const LaunchCfg& cfg, int max_n, size_t list_elems) {
+  const size_t smem = batched_smem_bytes(max_n, cfg.threads, FP64, list_elems);
   auto fn = md_batched_kernel<FP64, P, LSM, 2, MAXT>;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess)

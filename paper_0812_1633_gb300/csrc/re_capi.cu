@@ -379,6 +379,7 @@ int allocate(re_ctx* c) {
       (rc = dalloc(c, &s.fx, A)) || (rc = dalloc(c, &s.fy, A)) || (rc = dalloc(c, &s.fz, A)) ||
       (rc = dalloc(c, &s.rx, A)) || (rc = dalloc(c, &s.ry, A)) || (rc = dalloc(c, &s.rz, A)) ||
       (rc = dalloc(c, &s.ncnt, 8 * A)) || (rc = dalloc(c, &s.nbr, (size_t)c->n_nbr)) ||
+      (c->opt.path == RE_PATH_BATCHED && (rc = dalloc(c, &s.raw, (size_t)c->n_nbr))) ||
       (rc = dalloc(c, &s.T, R)) || (rc = dalloc(c, &s.U, R)) || (rc = dalloc(c, &s.K, R)) ||
       (rc = dalloc(c, &s.econs, R)) || (rc = dalloc(c, &s.vscale, R)) ||
       (rc = dalloc(c, &s.lam, R)) || (rc = dalloc(c, &s.fscale, R)) ||
@@ -477,7 +478,7 @@ size_t list_elems_for(const re_ctx* c, const LaunchCfg& k, const Scope& sc) {
     const size_t per = (size_t)(e.N + k.cluster - 1) / k.cluster;
     elems = std::max(elems, per * k.atom_threads * (size_t)e.capsub[pidx]);
   }
-  const size_t smem = re::batched_smem_bytes(sc.max_n, sc.max_ncell, k.threads,
+  const size_t smem = re::batched_smem_bytes(sc.max_n, k.threads,
                                              c->opt.precision == RE_PREC_FP64, elems);
   return smem + re::kBatchedStaticSmem <= (size_t)max_smem_optin() ? elems : 0;
 }
@@ -502,8 +503,8 @@ int check_cfg(re_ctx* c, const LaunchCfg& k, const Scope& sc) {
       k.threads < k.atom_threads * ((sc.max_n + k.cluster - 1) / k.cluster))
     return fail(c, RE_EINVAL, "%d atoms per CTA x %d threads per atom exceed 1024 threads; "
                 "use more CTAs per replica", (sc.max_n + k.cluster - 1) / k.cluster, k.atom_threads);
-  const size_t smem = re::batched_smem_bytes(sc.max_n, sc.max_ncell, k.threads,
-                                             c->opt.precision == RE_PREC_FP64, 0) +
+  const size_t smem = re::batched_admission_bytes(sc.max_n, sc.max_ncell, k.threads,
+                                                  c->opt.precision == RE_PREC_FP64) +
                       re::kBatchedStaticSmem;
   const int maxsm = max_smem_optin();
   if (smem > (size_t)maxsm)
@@ -555,7 +556,7 @@ int launch_class(re_ctx* c, int e, const int32_t* d_budget, cudaStream_t st, boo
   }
   cudaError_t err = re::launch_batched(c->s, c->d_ens, c->d_rep, work, c->ens[e].R, d_budget,
                                        c->opt.precision == RE_PREC_FP64, k, sc.max_n,
-                                       sc.max_ncell, list_elems_for(c, k, sc), 0, st, nullptr);
+                                       list_elems_for(c, k, sc), 0, st, nullptr);
   if (err != cudaSuccess) return cuda_fail(c, err, "batched MD launch (ensemble class)");
   return RE_OK;
 }
@@ -584,11 +585,11 @@ int relayout_lists(re_ctx* c, int mode) {
     }
   } else if (mode == 2) {
     cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work, c->n_rep, c->d_zero,
-                                       fp64, c->fcfg, c->max_n, c->max_ncell, 0, 0, c->stream);
+                                       fp64, c->fcfg, c->max_n, 0, 0, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
   } else {
     cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work, c->n_rep, c->d_zero,
-                                       fp64, c->cfg, c->max_n, c->max_ncell, 0, 0, c->stream);
+                                       fp64, c->cfg, c->max_n, 0, 0, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
   }
   RE_CUDA(c, cudaMemcpyAsync(c->s.nreb, c->d_io, 8 * R, cudaMemcpyDeviceToDevice, c->stream),
@@ -651,11 +652,11 @@ int launch_advance(re_ctx* c, const int32_t* d_budget, const int32_t* h_budget,
       RE_CUDA(c, cudaEventRecord(c->ev_fork, c->stream), "fork");
       RE_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0), "fork");
       cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work2 + nn, nw, d_budget,
-                                         fp64, wk, c->max_n, c->max_ncell, list_elems_for(c, wk),
+                                         fp64, wk, c->max_n, list_elems_for(c, wk),
                                          0, c->side, nullptr);
       if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch (wide class)");
       e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work2, nn, d_budget, fp64, c->cfg,
-                             c->max_n, c->max_ncell, list_elems_for(c, c->cfg), 0, c->stream,
+                             c->max_n, list_elems_for(c, c->cfg), 0, c->stream,
                              nullptr);
       if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
       RE_CUDA(c, cudaEventRecord(c->ev_join, c->side), "join");
@@ -670,7 +671,7 @@ int launch_advance(re_ctx* c, const int32_t* d_budget, const int32_t* h_budget,
                                        c->stream), "order work");
     const LaunchCfg& k = (!budgets && fr && fr->nx > 0 && c->use_fcfg) ? c->fcfg : c->cfg;
     cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, order ? c->d_work_ord : c->d_work,
-                                       c->n_rep, d_budget, fp64, k, c->max_n, c->max_ncell,
+                                       c->n_rep, d_budget, fp64, k, c->max_n,
                                        budgets ? list_elems_for(c, k) : 0, async_nx,
                                        c->stream, fr);
     if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
@@ -1067,7 +1068,7 @@ int free_shape(re_ctx* c, bool* narrower) {
   const bool fp64 = c->opt.precision == RE_PREC_FP64;
   *narrower = false;
   if (c->resident_clusters < 0)
-    c->resident_clusters = re::batched_max_active_clusters(fp64, c->cfg, c->max_n, c->max_ncell);
+    c->resident_clusters = re::batched_max_active_clusters(fp64, c->cfg, c->max_n);
   if (c->n_rep <= c->resident_clusters) return RE_OK;
   const std::string err = c->err;
   const int clusters[5] = {8, 4, 3, 2, 1};
@@ -1080,7 +1081,7 @@ int free_shape(re_ctx* c, bool* narrower) {
         if (pass == 0 ? p != c->cfg.atom_threads : p >= c->cfg.atom_threads) continue;
         LaunchCfg k{cl, threads_for(c->max_n, cl, p), c->cfg.cell_div, p, 0, 0, 0, 0, 0};
         if (k.threads > 1024 || check_cfg(c, k) != RE_OK) continue;
-        if (re::batched_max_active_clusters(fp64, k, c->max_n, c->max_ncell) < c->n_rep) continue;
+        if (re::batched_max_active_clusters(fp64, k, c->max_n) < c->n_rep) continue;
         c->err = err;
         c->fcfg = k;
         *narrower = true;

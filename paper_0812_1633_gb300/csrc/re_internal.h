@@ -95,6 +95,7 @@ struct StateDev {
   uint32_t *rx, *ry, *rz;
   int32_t* ncnt;
   uint16_t* nbr;
+  uint16_t* raw;  // as nbr: candidates that passed a list build's screening (scratch)
   double *T, *U, *K, *econs, *vscale;
   double *lam, *fscale;  // per replica: potential scale; pending force factor (null: 1)
   int64_t *step, *nreb;
@@ -171,7 +172,12 @@ void finish_ens(EnsDev& e);
 // Host-side launchers (re_kernels.cu).  All return the launch status.
 cudaError_t launch_init_lattice(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                                 int n_rep, int max_threads, cudaStream_t st);
-size_t batched_smem_bytes(int max_n, int max_ncell, int threads, bool fp64, size_t list_elems);
+size_t batched_smem_bytes(int max_n, int threads, bool fp64, size_t list_elems);
+// Admission of a replica of max_n atoms: the largest replicas that the batched
+// path takes and is tested for, as the bytes of a layout that holds a
+// cell-sorted copy of the positions and the cell tables beside the rest (the
+// kernel itself needs less, see batched_layout).
+size_t batched_admission_bytes(int max_n, int max_ncell, int threads, bool fp64);
 // Shared memory the batched kernel declares statically (replica constants and
 // hand-over words), reserved on top of batched_smem_bytes; launches check it.
 constexpr size_t kBatchedStaticSmem = 512;
@@ -185,18 +191,18 @@ constexpr size_t kBatchedStaticSmem = 512;
 // list_elems == 0 (lists in global memory).
 cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                            const int* d_work, int n_work, const int32_t* d_budget, bool fp64,
-                           const LaunchCfg& cfg, int max_n, int max_ncell, size_t list_elems,
+                           const LaunchCfg& cfg, int max_n, size_t list_elems,
                            int async_nx, cudaStream_t st, const FreeDev* fr = nullptr);
 // Clusters of the batched kernel that can be resident at once with this
 // launch shape (0 when the query fails).
-int batched_max_active_clusters(bool fp64, const LaunchCfg& cfg, int max_n, int max_ncell);
+int batched_max_active_clusters(bool fp64, const LaunchCfg& cfg, int max_n);
 
 // One instantiation of the batched kernel (precision, threads per atom, list
 // placement, mode) and its launch; defined in re_batched.cuh, instantiated in
 // the re_batched_*.cu translation units.
 #define BATCHED_LAUNCH_ARGS                                                               \
   const StateDev &s, const EnsDev *d_ens, const RepDev *d_rep, const int *d_work,        \
-      int n_work, const int32_t *d_budget, const LaunchCfg &cfg, int max_n, int max_ncell, \
+      int n_work, const int32_t *d_budget, const LaunchCfg &cfg, int max_n, \
       size_t list_elems, int async_nx, cudaStream_t st, const FreeDev *fr
 // MAXT: 1024, or kNarrowThreads for launches of at most that many threads
 // per CTA (a larger register budget per thread).
@@ -204,7 +210,7 @@ constexpr int kNarrowThreads = 896;
 template <bool FP64, int P, bool LSM, int MODE, int MAXT>
 cudaError_t launch_batched_t(BATCHED_LAUNCH_ARGS);
 template <bool FP64, int P, bool LSM, int MAXT>
-int max_active_clusters_t(const LaunchCfg& cfg, int max_n, int max_ncell, size_t list_elems);
+int max_active_clusters_t(const LaunchCfg& cfg, int max_n, size_t list_elems);
 // Work lists of a split launch: replicas ranked by decreasing temperature T
 // (ties by index); the wide_n hottest go to work[R - wide_n .. R), in rank
 // order, the others to work[0 .. R - wide_n).  One ensemble of R replicas.

@@ -180,7 +180,7 @@ __global__ void plain_rebuild(StateDev S, const EnsDev* __restrict__ ens,
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int g = rd.atom_off + i;
     S.ncnt[(size_t)rd.atom_off * 8 + i] =
-        build_sublist<1>(i, 0, hi_of, N, E.nc, E.m, cstart, spos, K.rl2u, nb, (uint32_t)i,
+        build_sublist_cells<1>(i, 0, hi_of, N, E.nc, E.m, cstart, spos, K.rl2u, nb, (uint32_t)i,
                          (uint32_t)N, E.capsub[0], &overflow);
     S.rx[g] = hp[i].x;
     S.ry[g] = hp[i].y;
@@ -865,16 +865,24 @@ cudaError_t launch_init_lattice(const StateDev& s, const EnsDev* d_ens, const Re
   return cudaGetLastError();
 }
 
-size_t batched_smem_bytes(int max_n, int max_ncell, int threads, bool fp64, size_t list_elems) {
-  return batched_layout(max_n, max_ncell, threads, fp64, list_elems, nullptr, nullptr);
+size_t batched_smem_bytes(int max_n, int threads, bool fp64, size_t list_elems) {
+  return batched_layout(max_n, threads, fp64, list_elems, nullptr, nullptr);
+}
+
+size_t batched_admission_bytes(int max_n, int max_ncell, int threads, bool fp64) {
+  const size_t n = (size_t)max_n, t = (size_t)threads;
+  const size_t fixed = 2 * kNoiseChunk * kSvrStepBytes + 12 * kNoiseChunk +
+                       kMaxCluster * kMaxWarps * 20 + kMaxCluster * 4 + 256;
+  return fixed + n * (fp64 ? 48 : 32) + (fp64 ? 0 : 12 * t) + 8 * ((size_t)max_ncell + 1) +
+         std::max(14 * t + 8, 2 * n);
 }
 
 
-int batched_max_active_clusters(bool fp64, const LaunchCfg& cfg, int max_n, int max_ncell) {
+int batched_max_active_clusters(bool fp64, const LaunchCfg& cfg, int max_n) {
 #define RE_MC(F, PP)                                                                   \
   return cfg.threads <= kNarrowThreads                                                   \
-             ? max_active_clusters_t<F, PP, false, kNarrowThreads>(cfg, max_n, max_ncell, 0) \
-             : max_active_clusters_t<F, PP, false, 1024>(cfg, max_n, max_ncell, 0);
+             ? max_active_clusters_t<F, PP, false, kNarrowThreads>(cfg, max_n, 0) \
+             : max_active_clusters_t<F, PP, false, 1024>(cfg, max_n, 0);
 #define RE_MCP(F)             \
   switch (cfg.atom_threads) { \
     case 1: RE_MC(F, 1)       \
@@ -971,7 +979,7 @@ cudaError_t launch_attempt_add(const StateDev& s, int n_ens, int n, cudaStream_t
 
 cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                            const int* d_work, int n_work, const int32_t* d_budget, bool fp64,
-                           const LaunchCfg& cfg, int max_n, int max_ncell, size_t list_elems,
+                           const LaunchCfg& cfg, int max_n, size_t list_elems,
                            int async_nx, cudaStream_t st, const FreeDev* fr) {
   if (n_work <= 0) return cudaSuccess;
   const bool lsm = list_elems > 0;
@@ -981,10 +989,10 @@ cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev*
 #define RE_LB(F, PP, LS, M)                                                                   \
   return cfg.threads <= kNarrowThreads                                                         \
              ? launch_batched_t<F, PP, LS, M, kNarrowThreads>(s, d_ens, d_rep, d_work, n_work, \
-                                                              d_budget, cfg, max_n, max_ncell, \
+                                                              d_budget, cfg, max_n,            \
                                                               list_elems, async_nx, st, fr)    \
              : launch_batched_t<F, PP, LS, M, 1024>(s, d_ens, d_rep, d_work, n_work, d_budget, \
-                                                    cfg, max_n, max_ncell, list_elems,         \
+                                                    cfg, max_n, list_elems,                    \
                                                     async_nx, st, fr);
 #define RE_LBP(F, LS, M)                           \
   switch (cfg.atom_threads) {                      \

@@ -4,6 +4,7 @@
 // and the free-running exchange protocol.  Internal header.
 #pragma once
 #include <cooperative_groups.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 
@@ -222,26 +223,24 @@ struct Pos64 {
 struct BatchedSmem {
   uint16_t* nb_sm;  // this CTA's neighbour sub-lists when they fit in shared memory
   void* pos;       // uint4[N] (mixed: top 32 bits of x, y, z) or Pos64[N] (fp64)
-  int* cstart;     // ncell + 1
-  int* ccnt;       // ncell
-  uint4* spos;     // cell-sorted positions (.w = atom index)
-  int* wscan;      // 2 x (threads + 1): block scan of own atoms in cell order
-  uint16_t* own_sorted;  // threads: sorted slots of this CTA's atoms
-  int* cnt_sh;     // threads: sub-list counts handed to the owners
+  uint4* hk;       // f16 screening vectors of the atoms, rows of 32 (list build)
+  uint2* box;      // bounding box of each row: centre bytes, half-width bytes
+  uint8_t* act;    // per warp: the rows in reach of its atoms
   uint32_t* ref;     // 3 per own atom: top 32 bits of the coordinates at the last list build
   long long* rec_k;  // kNoiseChunk: 2K of each step (fixed point), CTA 0
   float* rec_e;      // kNoiseChunk: alpha - 1 of each step
-  uint16_t* acell;
   double2* noise;  // 2 x kNoiseChunk thermostat records (double buffered)
   float* slot_md;  // [cluster][warps]
   double* slot_uk; // [cluster][warps][2]
   int* slot_st;    // [cluster]
-  int* iscr;       // 64
 };
 
 __host__ __device__ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-__host__ __device__ inline size_t batched_layout(int max_n, int max_ncell, int threads, bool fp64,
+// A warp's list of rows (of 32 atoms), with room for four more.
+__host__ __device__ inline size_t row_list_bytes(int n) { return (size_t)((n + 31) / 32 + 11) / 8 * 8; }
+
+__host__ __device__ inline size_t batched_layout(int max_n, int threads, bool fp64,
                                                  size_t list_elems, unsigned char* base,
                                                  BatchedSmem* out) {
   size_t off = 0;
@@ -251,27 +250,19 @@ __host__ __device__ inline size_t batched_layout(int max_n, int max_ncell, int t
     off += bytes;
     return o;
   };
+  const size_t o_pos = take((size_t)max_n * (fp64 ? 32 : 16), 32);  // at the base: fixed offset
   const size_t o_nbs = take(list_elems * 2, 16);
-  const size_t o_pos = take((size_t)max_n * (fp64 ? 32 : 16), 32);
-  const size_t o_sp = take((size_t)max_n * 16, 16);
+  const size_t rows = ((size_t)max_n + 31) / 32;  // of 32 atoms
+  const size_t o_hk = take(rows * 512, 128);
+  const size_t o_bx = take(rows * sizeof(uint2), 8);
+  const size_t o_ar = take((size_t)kMaxWarps * row_list_bytes(max_n), 8);
   const size_t o_noise = take((size_t)kNoiseChunk * 2 * kSvrStepBytes, 16);
   const size_t o_uk = take((size_t)kMaxCluster * kMaxWarps * 2 * 8, 16);
   const size_t o_md = take((size_t)kMaxCluster * kMaxWarps * 4, 4);
   const size_t o_st = take(kMaxCluster * 4, 4);
-  const size_t o_isc = take(64 * 4, 4);
   const size_t o_ref = take(fp64 ? 0 : (size_t)threads * 3 * 4, 4);  // own atoms <= threads
   const size_t o_rk = take((size_t)kNoiseChunk * 8, 8);
   const size_t o_re = take((size_t)kNoiseChunk * 4, 4);
-  const size_t o_cs = take((size_t)(max_ncell + 1) * 4, 4);
-  const size_t o_cc = take((size_t)(max_ncell + 1) * 4, 4);
-  // one region, two lifetimes: the atoms' cell ids during the cell sort, then
-  // the block scan, the own-slot list and the hand-over counts of the list build
-  const size_t scan_bytes = (size_t)2 * (threads + 1) * 4 + (size_t)threads * 4 + (size_t)threads * 2;
-  const size_t o_un = take(scan_bytes > (size_t)max_n * 2 ? scan_bytes : (size_t)max_n * 2, 4);
-  const size_t o_ws = o_un;
-  const size_t o_cn = o_un + (size_t)2 * (threads + 1) * 4;
-  const size_t o_os = o_cn + (size_t)threads * 4;
-  const size_t o_ac = o_un;
   if (out) {
     out->nb_sm = reinterpret_cast<uint16_t*>(base + o_nbs);
     out->pos = base + o_pos;
@@ -279,23 +270,18 @@ __host__ __device__ inline size_t batched_layout(int max_n, int max_ncell, int t
     out->slot_uk = reinterpret_cast<double*>(base + o_uk);
     out->slot_md = reinterpret_cast<float*>(base + o_md);
     out->slot_st = reinterpret_cast<int*>(base + o_st);
-    out->iscr = reinterpret_cast<int*>(base + o_isc);
     out->ref = reinterpret_cast<uint32_t*>(base + o_ref);
     out->rec_k = reinterpret_cast<long long*>(base + o_rk);
     out->rec_e = reinterpret_cast<float*>(base + o_re);
-    out->cstart = reinterpret_cast<int*>(base + o_cs);
-    out->ccnt = reinterpret_cast<int*>(base + o_cc);
-    out->spos = reinterpret_cast<uint4*>(base + o_sp);
-    out->wscan = reinterpret_cast<int*>(base + o_ws);
-    out->cnt_sh = reinterpret_cast<int*>(base + o_cn);
-    out->own_sorted = reinterpret_cast<uint16_t*>(base + o_os);
-    out->acell = reinterpret_cast<uint16_t*>(base + o_ac);
+    out->hk = reinterpret_cast<uint4*>(base + o_hk);
+    out->box = reinterpret_cast<uint2*>(base + o_bx);
+    out->act = reinterpret_cast<uint8_t*>(base + o_ar);
   }
   return align_up(off, 128);
 }
 
 struct KernelDims {
-  int max_n, max_ncell;
+  int max_n;
   size_t list_elems;  // shared-memory list entries per CTA (0: lists in global memory)
   int async_nx;       // > 0: free-running mode with this many master steps
 };
@@ -322,7 +308,7 @@ __device__ __forceinline__ uint32_t* rcomp(const StateDev& S, int d) {
 // The sub-list of column `col` of a list with `ncols` columns: entry k at
 // element ((k / 4) * ncols + col) * 4 + k % 4 of nb.
 template <int P, class PosFn>
-__device__ int build_sublist(int i, int q, PosFn pos_hi, int N, int nc, int m, const int* cstart,
+__device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, int m, const int* cstart,
                              const uint4* spos, float rl2u, uint16_t* nb, uint32_t col,
                              uint32_t ncols, int cap_sub, int* overflow) {
   const Hi3 pi = pos_hi(i);
@@ -395,6 +381,323 @@ __device__ int build_sublist(int i, int q, PosFn pos_hi, int N, int nc, int m, c
   // pad to a whole block of four with the atom's own index (skipped by r2 > 0)
   for (int k = cnt; k & 3; ++k) nb[wofs++] = (uint16_t)i;
   return cnt;
+}
+
+// ------------------------------------------------- list build, batched kernel
+// Which atoms lie within the list radius of which is first screened on the
+// tensor cores: with a = 2 pi / L,
+//   S = sum over d of cos(a dx_d) = sum of cos a x_d cos a x'_d + sin a x_d sin a x'_d
+// is a dot product of two six-vectors, periodic by itself, and within a
+// distance r it is at least 3 cos(a r / sqrt 3) (cos(a sqrt u) is convex in u,
+// so the least sum at a given r^2 is the one of equal components).  One
+// mma.m16n8k8 (f16 vectors, f32 sums; the other two of its eight products add
+// the limit, and put the last row's missing atoms beyond it) screens 16 atoms against 8; one funnel shift per result collects
+// its sign.  Of the candidates that pass (7 to 20 % more than the list at
+// L = 17 to 10) the exact test on the 32-bit positions keeps the list, so the
+// pair set does not depend on the screening.  No cells are built or sorted: a
+// warp goes through the rows (32 consecutive atoms) whose bounding box lies
+// within the list radius of its own atoms' box.  Atoms are renumbered in space
+// order from time to time, so both boxes are small; the order affects the time
+// only.
+//
+// A lane's hits come unevenly from mask to mask, but in all the lanes of a warp
+// have nearly the same number.  So the masks are only noted, and the loop over
+// their bits, with the exact test, lets every lane go through its own notes at
+// its own pace: as many turns as the fullest lane has hits (emptying mask by
+// mask takes three times as many).  Bound by instruction issue.  A build took,
+// against the cell scan it replaces, in thousand clocks: 53 against 74 (864
+// atoms on two CTAs, skin 0.3), 162 against 175 (2048, skin 0.5), 189 against
+// 440 (4000 on four); 14, 55 and 77 of them screen, the rest is the exact test.
+
+__device__ __forceinline__ uint32_t pack8(Hi3 p) {
+  return (p.x >> 24) | ((p.y >> 24) << 8) | ((p.z >> 24) << 16);
+}
+
+// Bounding box of the bytes of a warp's values w (those with `in`): centre and
+// half-width bytes of the interval of every coordinate around one of them.
+__device__ __forceinline__ uint2 warp_box(uint32_t w, bool in) {
+  const uint32_t ref = __shfl_sync(0xffffffffu, w, __ffs(__ballot_sync(0xffffffffu, in)) - 1);
+  uint32_t cen = 0, half = 0;
+#pragma unroll
+  for (int d = 0; d < 24; d += 8) {
+    const int e = in ? (int)(int8_t)((w >> d) - (ref >> d)) : 0;
+    const int l = __reduce_min_sync(0xffffffffu, e), h = __reduce_max_sync(0xffffffffu, e);
+    const int m = (l + h) >> 1;
+    cen |= (((ref >> d) + (uint32_t)m) & 255u) << d;
+    half |= (uint32_t)(h - m) << d;
+  }
+  return make_uint2(cen, half);
+}
+
+__device__ __forceinline__ uint32_t half2_bits(float lo, float hi) {
+  const __half2 h = __floats2half2_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// Screening vectors and row boxes of all N atoms (whole block): atom j's
+// (cx, cy, cz, sx, sy, sz, 0, 1) at hk[j].  Ends with a block barrier.
+template <class PosFn>
+__device__ __forceinline__ void cta_screen_vectors(PosFn pos_hi, int N, uint4* hk, uint2* box) {
+  const int T = blockDim.x, lane = threadIdx.x & 31;
+  constexpr float kTurn = 1.4629180792671596e-09f;  // 2 pi / 2^32
+  for (int r = threadIdx.x >> 5; r < (N + 31) / 32; r += T >> 5) {
+    const int j = r * 32 + lane;
+    const Hi3 p = j < N ? pos_hi(j) : Hi3{0u, 0u, 0u};
+    // signed: angles in [-pi, pi], where the fast functions are accurate
+    const float ax = (float)(int)p.x * kTurn, ay = (float)(int)p.y * kTurn, az = (float)(int)p.z * kTurn;
+    hk[j] = make_uint4(half2_bits(__cosf(ax), __cosf(ay)), half2_bits(__cosf(az), __sinf(ax)),
+                       half2_bits(__sinf(ay), __sinf(az)), j < N ? 0x3C000000u : 0x3C007800u);
+    const uint2 b = warp_box(pack8(p), j < N);
+    if (lane == 0) box[r] = b;
+  }
+  __syncthreads();
+}
+
+// The end of a sub-list: overflow and coincident atoms (closer than L / 2^32:
+// the pair loop cannot give their force a direction) reported, the last block
+// filled up with the atom's own index.
+__device__ __forceinline__ int finish_sublist(int cnt, uint2 blk, uint2* out, int i,
+                                              bool coincident, int cap_sub, int* overflow) {
+  if (coincident) *overflow |= kStNumeric;
+  if (cnt > cap_sub) {
+    *overflow |= kStOverflow;
+    return cap_sub;  // whole blocks
+  }
+  if (cnt & 3) {
+    for (int k = cnt; k & 3; ++k) {
+      blk.x = __funnelshift_r(blk.x, blk.y, 16);
+      blk.y = __byte_perm(blk.y, (uint32_t)i, 0x5432);
+    }
+    *out = blk;
+  }
+  return cnt;
+}
+
+// The list of a small replica, by testing every atom: lane q takes the atoms j
+// with j % P == q, in increasing order.  Below kDirectBuild atoms a lane this
+// costs less than the screening and its notes (20 instructions an atom, no
+// divergence): with P = 4 at 500 atoms 19.6 thousand clocks a build against
+// 23.5; with P = 2 at 864 atoms, past the line, 58 against 53.
+constexpr int kDirectBuild = 256;
+
+template <int P, class PosFn>
+__device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosFn pos_hi, int N,
+                                                    float rl2u, uint16_t* nb, uint32_t col,
+                                                    uint32_t ncols, int cap_sub, int* overflow) {
+  if (!own) return 0;
+  const Hi3 pi = pos_hi(i);
+  int cnt = 0;
+  uint2 blk = make_uint2(0u, 0u);  // the last four entries
+  uint2* out = reinterpret_cast<uint2*>(nb) + col;
+  bool coincident = false;
+#pragma unroll 4
+  for (int j = q; j < N; j += P) {
+    const float r2 = sep2_hi(pi, pos_hi(j));
+    const bool add = r2 < rl2u && j != i;
+    coincident |= add && r2 == 0.0f;
+    if (add) {
+      blk.x = __funnelshift_r(blk.x, blk.y, 16);
+      blk.y = __byte_perm(blk.y, (uint32_t)j, 0x5432);
+    }
+    const bool full = add && (cnt & 3) == 3;
+    if (full && cnt < cap_sub) *out = blk;
+    if (full) out += ncols;
+    cnt += add ? 1 : 0;
+  }
+  return finish_sublist(cnt, blk, out, i, coincident, cap_sub, overflow);
+}
+
+// Sub-list of lane q (of P) of atom i, by whole warps (every lane of the warp
+// calls; `own` says whether it holds an atom; iw: the warp's first atom): entry
+// k at element ((k / 4) * ncols + col) * 4 + k % 4 of nb, written four at a
+// time, the last four filled up with the atom's own index.  raw, rcol, rncols:
+// room for the notes, one 8-byte word each, laid out likewise.  act: this warp's
+// row list.
+//
+// Tile v of a row (v = 0..3) holds the atoms t + 8 v + 4 c at columns 2 t + c,
+// and lane 4 g + t gets columns 2 t, 2 t + 1 of the tile rows g and g + 8: it
+// sees the row's atoms j with j % 4 == t, in increasing order.  Tile rows are
+// the warp's atoms so placed that the four lanes 4 g + t own the atoms of the
+// rows g, g + 8 (of one tile, or two for P = 1); they swap their masks so that
+// each keeps its own atom's.  Neighbouring atoms go to different lanes of an
+// atom: its sub-lists are nearly equal.  The order of a sub-list (by row, then
+// column, then tile) depends on the atom and P alone, so that the FP32 sums, and
+// with them the trajectories, do not change with the cluster size.
+template <int P, class PosFn>
+__device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_hi, int N,
+                                             const uint4* hk, const uint2* box, uint8_t* act,
+                                             float rl2u, uint16_t* nb, uint32_t col,
+                                             uint32_t ncols, uint16_t* raw, uint32_t rcol,
+                                             uint32_t rncols, int cap_sub, int* overflow) {
+  const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
+  if (!__any_sync(0xffffffffu, own)) return 0;
+  const Hi3 pi = own ? pos_hi(i) : Hi3{0u, 0u, 0u};
+  // the rows in reach: gap between the boxes, in units of L / 256 (a byte
+  // stands for a unit's width)
+  const float rl = sqrtf(rl2u);
+  int nact = 0;
+  {
+    const uint2 mine = warp_box(pack8(pi), own);
+    const float r8 = rl * 5.9604644775390625e-08f;
+    const int gap_max = (int)ceilf(r8 * r8) + 1;
+    const int nrow = (N + 31) / 32;
+    for (int r0 = 0; r0 < nrow; r0 += 32) {
+      bool near = false;
+      if (r0 + lane < nrow) {
+        const uint2 b = box[r0 + lane];
+        int g2 = 0;
+#pragma unroll
+        for (int d = 0; d < 24; d += 8) {
+          const int e = abs((int)(int8_t)((b.x >> d) - (mine.x >> d)));
+          const int gap = max(0, e - (int)((b.y >> d) & 255u) - (int)((mine.y >> d) & 255u) - 1);
+          g2 += gap * gap;
+        }
+        near = g2 <= gap_max;
+      }
+      const uint32_t bal = __ballot_sync(0xffffffffu, near);
+      if (near) act[nact + __popc(bal & ((1u << lane) - 1u))] = (uint8_t)(r0 + lane);
+      nact += __popc(bal);
+    }
+    if (lane < 4) act[nact + lane] = 0;  // for the rest of the last four
+    __syncwarp();
+  }
+  // tile rows: minus the atoms' vectors, 1 and the limit.  Below it by 2.2e-3:
+  // each of the twelve f16 values is off by at most 2^-12, which moves S by at
+  // most 6 sqrt 2 2^-12 = 2.1e-3
+  constexpr int NT = P == 1 ? 2 : 1;  // tiles
+  uint32_t A[NT][2];
+  {
+    const float lim = 3.0f * __cosf(rl * (1.4629180792671596e-09f * 0.57735026918962576f)) - 2.2e-3f;
+    const uint32_t lim2 = 0x3C00u | ((uint32_t)__half_as_ushort(__float2half_rd(lim)) << 16);
+    const uint32_t* h = reinterpret_cast<const uint32_t*>(hk);
+#pragma unroll
+    for (int k = 0; k < NT; ++k)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int a = P == 1 ? 4 * g + 2 * k + u : (P == 2 ? 2 * g + u : (P == 4 ? g : g >> 1));
+        A[k][u] = t == 3 ? lim2 : h[min(iw + a, N - 1) * 4 + t] ^ 0x80008000u;
+      }
+  }
+  int cnt = 0, nm = 0;             // entries, notes
+  uint2 blk = make_uint2(0u, 0u);  // the last four entries
+  uint2* out = reinterpret_cast<uint2*>(nb) + col;
+  uint2* const rawp = reinterpret_cast<uint2*>(raw) + rcol;
+  int zeros = 0;
+  // the exact test of the candidates noted so far (whole warps; without
+  // branches: a lane that has none left tests something, and keeps nothing).
+  // Bit 31 - k of a note's mask .x stands for an atom 4 (k % 8) + column of the
+  // row in byte k / 8 of .y.
+  auto drain = [&]() {
+    uint2 cur = make_uint2(0u, 0u), next = cur;
+    if (nm > 0) cur = rawp[0];
+    if (nm > 1) next = rawp[rncols];
+    int left = nm - 1;  // notes after `cur`
+    const uint2* in = rawp + 2 * (size_t)rncols;
+    while (__any_sync(0xffffffffu, cur.x != 0u)) {
+      const uint32_t k = (uint32_t)__clz(cur.x) & 31u;
+      const uint32_t column = P == 1 ? k >> 3 : (P == 2 ? (uint32_t)(t & 1) + ((k >> 2) & 2u) : (uint32_t)t);
+      const uint32_t j = ((cur.y >> (k & 24u)) & 255u) * 32u + (k & 7u) * 4u + column;
+      const float r2 = sep2_hi(pi, pos_hi((int)j));
+      const bool in_list = cur.x != 0u && r2 < rl2u;
+      const bool zero = in_list && r2 == 0.0f;  // the atom itself, or another at the same point
+      const bool add = in_list && !zero;
+      zeros += zero ? 1 : 0;
+      cur.x &= ~(0x80000000u >> k);
+      if (add) {
+        blk.x = __funnelshift_r(blk.x, blk.y, 16);
+        blk.y = __byte_perm(blk.y, j, 0x5432);
+      }
+      const bool full = add && (cnt & 3) == 3;
+      if (full && cnt < cap_sub) *out = blk;
+      if (full) out += ncols;
+      cnt += add ? 1 : 0;
+      const bool turn = cur.x == 0u && left > 0;
+      if (turn) cur = next;
+      left -= turn ? 1 : 0;
+      if (turn && left > 0) next = *in;
+      if (turn) in += rncols;
+    }
+    nm = 0;
+  };
+  const uint32_t hk_lane = (uint32_t)__cvta_generic_to_shared(hk) +
+                           (uint32_t)(((lane & 7) >> 1) + (lane & 24) + 4 * (lane & 1)) * 16u;
+  constexpr int NM = P == 1 ? 4 : (P == 2 ? 2 : 1);  // masks a lane keeps of four rows
+  for (int a0 = 0; a0 < nact; a0 += 4) {
+    uint32_t m[2 * NT] = {};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      uint32_t b[4];
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                   : "r"(hk_lane + (uint32_t)act[a0 + u] * 512u)
+                   : "memory");
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+          float c0, c1, c2, c3;
+          asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, "
+              "{%7, %7, %7, %7};"
+              : "=f"(c0), "=f"(c1), "=f"(c2), "=f"(c3)
+              : "r"(A[k][0]), "r"(A[k][1]), "r"(b[v]), "f"(0.0f));
+          m[2 * k] = __funnelshift_l(__float_as_uint(c0), m[2 * k], 1);
+          m[2 * k] = __funnelshift_l(__float_as_uint(c1), m[2 * k], 1);
+          if (P <= 2) {
+            m[2 * k + 1] = __funnelshift_l(__float_as_uint(c2), m[2 * k + 1], 1);
+            m[2 * k + 1] = __funnelshift_l(__float_as_uint(c3), m[2 * k + 1], 1);
+          }
+        }
+    }
+    // each lane's own atom's masks (a byte a row, the first row on top): of the
+    // columns t, and of the columns t ^ 1, t ^ 2, t ^ 3 (P = 1) or t ^ 2 (P = 2).
+    // Nothing of rows past the last one, nothing for lanes without an atom
+    const uint32_t valid = !own ? 0u : (nact - a0 >= 4 ? 0xffffffffu : ~(0xffffffffu >> (8 * (nact - a0))));
+    uint32_t mk[NM];
+    if (P == 1) {
+      uint32_t w[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int want = t ^ x;  // the lane that this one gives to owns row `want`
+        const uint32_t give = want & 2 ? (want & 1 ? m[2 * NT - 1] : m[2 * NT - 2])
+                                       : (want & 1 ? m[1] : m[0]);
+        w[x] = (x == 0 ? give : __shfl_xor_sync(0xffffffffu, give, x)) & valid;
+      }
+      // a note a row, the columns 0..3 from the top byte down
+      const uint32_t l0 = __byte_perm(w[0], w[1], 0x5140), l1 = __byte_perm(w[2], w[3], 0x5140),
+                     h0 = __byte_perm(w[0], w[1], 0x7362), h1 = __byte_perm(w[2], w[3], 0x7362);
+      const uint32_t order = 0x3210u ^ ((uint32_t)(t ^ 3) * 0x1111u);
+      mk[0] = __byte_perm(__byte_perm(h0, h1, 0x7632), 0, order);
+      mk[1 % NM] = __byte_perm(__byte_perm(h0, h1, 0x5410), 0, order);
+      mk[2 % NM] = __byte_perm(__byte_perm(l0, l1, 0x7632), 0, order);
+      mk[3 % NM] = __byte_perm(__byte_perm(l0, l1, 0x5410), 0, order);
+    } else if (P == 2) {
+      const uint32_t own_cols = (t & 2 ? m[1] : m[0]) & valid;
+      const uint32_t others = __shfl_xor_sync(0xffffffffu, t & 2 ? m[0] : m[1], 2) & valid;
+      const uint32_t c0 = t & 2 ? others : own_cols, c1 = t & 2 ? own_cols : others;
+      // a note two rows, of each the columns t & 1, then those two further
+      mk[0] = __byte_perm(c0, c1, 0x3726);
+      mk[NM - 1] = __byte_perm(c0, c1, 0x1504);
+    } else {
+      mk[0] = (P == 4 ? m[0] : m[0] & (g & 1 ? 0x33333333u : 0xCCCCCCCCu)) & valid;
+    }
+    const uint32_t rows4 = *reinterpret_cast<const uint32_t*>(act + a0);
+#pragma unroll 1
+    for (int x = 0; x < NM; ++x) {
+      const uint32_t w = mk[0];
+#pragma unroll
+      for (int y = 0; y + 1 < NM; ++y) mk[y] = mk[y + 1];
+      if (__any_sync(0xffffffffu, nm == cap_sub / 4)) drain();
+      // the row of each byte from the top, lowest byte first
+      const uint32_t sel = P == 1 ? x * 0x1111u : (P == 2 ? 0x1100u + x * 0x2222u : 0x3210u);
+      if (w) rawp[(size_t)nm++ * rncols] = make_uint2(w, __byte_perm(rows4, 0, sel));
+    }
+  }
+  drain();
+  if (!own) return 0;
+  // of the atom's lanes, the one whose columns hold the atom met it once
+  const bool self = P == 1 || (P == 2 && (t & 1) == (i & 1)) || (P == 4 && t == (i & 3)) ||
+                    (P == 8 && t == (i & 3) && (g & 1) == ((i >> 3) & 1));
+  return finish_sublist(cnt, blk, out, i, zeros > (self ? 1 : 0), cap_sub, overflow);
 }
 
 // Mixed-precision sub-list loop of lane (i, q); see mixed_pair.
