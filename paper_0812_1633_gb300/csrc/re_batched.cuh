@@ -278,16 +278,26 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       du = warp_sum(du);
       dk = warp_sum(dk);
     } else {
-      MixedAcc a{0.f, 0.f, 0.f, 0.f, 0, 0.f, 0};
+      PairAcc a{0ull, 0ull, 0ull, 0ull, 0ull, 3.0e38f};
       if (own) {
+        const uint4 pi = posm[i];
+        const Hi3 hi{pi.x, pi.y, pi.z};
         if (energy)
-          a = mixed_sublist_forces<true>(i, posm, nb, mycol, ncols, cnt, K);
+          a = mixed_sublist_forces<true>(hi, posm, nb, mycol, ncols, cnt, K);
         else
-          a = mixed_sublist_forces<false>(i, posm, nb, mycol, ncols, cnt, K);
+          a = mixed_sublist_forces<false>(hi, posm, nb, mycol, ncols, cnt, K);
       }
-      const float ax = group_sum<P>(a.fx), ay = group_sum<P>(a.fy), az = group_sum<P>(a.fz);
+      __syncwarp();
+      const bool near = a.tmin <= K.rc2u_hi - K.rc2u_lo;
+      if (energy)
+        mixed_cut_fix<true>(near, i, posm, nb, mycol, ncols, cnt, K, a);
+      else
+        mixed_cut_fix<false>(near, i, posm, nb, mycol, ncols, cnt, K, a);
+      const float ax = group_sum<P>(lo2(a.fx) + hi2(a.fx)), ay = group_sum<P>(lo2(a.fy) + hi2(a.fy)),
+                  az = group_sum<P>(lo2(a.fz) + hi2(a.fz));
       float ae = 0.0f;
-      if (energy) ae = group_sum<P>(a.e) - ucf * (float)group_sum<P>(a.nin);  // uniform flag
+      if (energy)  // uniform flag
+        ae = group_sum<P>(lo2(a.e) + hi2(a.e)) - ucf * group_sum<P>(lo2(a.n) + hi2(a.n));
       if (own) {
         if (!isfinite(ax) || !isfinite(ay) || !isfinite(az)) st |= kStNumeric;
         if (energy && q == 0) {

@@ -40,9 +40,11 @@ struct StepConst {
   double lam32, lam64, inv_l, dtq, hdt, inv_hdt, uc, rc2, c_th, kbar;
   double kbar1, af1, bf1, gf1;  // kbar = kbar1 T, af = af1 T, bf = bf1 sqrt(T), gf = gf1 / sqrt(T)
   double lamv;                  // the replica's potential scale (set_potential_scale)
+  double f24;                   // 24 kappa^4
   double rc2x;                  // rc^2 in units (L / 2^42)^2 (exact cutoff test, mixed path)
-  float hlf;                    // FP32 half-kick factor per force unit, times lamv
-  float rc2u, rl2u, half2u, inv_lam2;
+  float hlf;                    // FP32 half-kick factor per unit of the mixed pair sums, times lamv
+  float rc2u, rl2u, half2u;
+  float cs, c3;                 // mixed pair forces: cs = -2^k, c3 = 2 kappa^3, (2^32 / L)^2 = kappa 2^k
   float rc2u_lo, rc2u_hi;       // rc2u (1 -+ 2e-6): the band decided on 42-bit separations
   // thermostat constants of the mixed path (used in FP32): c - 1,
   // (1 - c) Kbar / Nf, 2 sqrt(c (1 - c) Kbar / Nf), sqrt(c Nf / ((1 - c) Kbar))
@@ -71,7 +73,8 @@ struct EnsDev : EnsHdr {
 // (its Hamiltonian is K + lam U_LJ: forces and U scale by lam).
 __host__ __device__ inline void set_potential_scale(StepConst& k, double lam) {
   k.lamv = lam;
-  k.hlf = (float)(k.hdt * k.lam32 * lam);
+  // the mixed pair sums are in units of 24 (2^k)^4 s^4 d, s = 1/r^2 in sigma units
+  k.hlf = (float)(k.hdt * k.lam32 * lam * k.f24);
 }
 
 // The constants of StepConst that depend on the target temperature T.

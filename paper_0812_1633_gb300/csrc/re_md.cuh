@@ -114,11 +114,17 @@ __device__ __forceinline__ float sep2_hi(Hi3 a, Hi3 b) {
 }
 
 // ------------------------------------------------------------------ forces
-// Mixed precision pair loop of atom i.  Separations are exact 32-bit integer
-// minimum images (units lam = L / 2^32) converted to FP32 once; the pair force
-// and energy are FP32; the per-atom sums are FP32 over this atom's list and
-// are folded into FP64 by the caller.  Force on i from j = fs * d with
-// fs = s^4 (24 - 48 s^3), s = 1/r^2 (sigma units); pair energy 4 s^3 (s^3 - 1).
+// Mixed precision pair forces.  Separations are exact 32-bit integer minimum
+// images (units lam = L / 2^32) converted to FP32 once; the pair force and
+// energy are FP32, and so are the sums over one sub-list.  Force on i from j =
+// fs * d with fs = s^4 (24 - 48 s^3), s = 1/r^2 (sigma units); pair energy
+// 4 s^3 (s^3 - 1).
+//
+// Two list entries are taken at a time, as packed f32x2 instructions (21
+// instead of 28 issued instructions per entry), without a branch per pair:
+// with q = -2 s^3 the force is fs = 24 s^4 (1 + q) (the factor 24 is part of
+// StepConst::hlf), multiplied by 1 inside the cutoff and 0 outside, and the
+// pair energy is q (q + 2).
 //
 // The cutoff test.  The force is truncated at rc (Example section), so it
 // jumps there by F(rc) ~ 0.04: a pair put on the wrong side of rc costs its
@@ -128,21 +134,55 @@ __device__ __forceinline__ float sep2_hi(Hi3 a, Hi3 b) {
 // pair outside a relative band of 2e-6 around rc^2, and pairs inside the band
 // are decided in FP64 on 42-bit separations: the top 32 bits and the next 10
 // bits of each coordinate (kept in .w of the shared-memory position, 10 bits
-// per coordinate).  The result equals the FP64 test on the full positions
-// except for pairs within ~1e-11 of rc.
-struct MixedAcc {
-  float fx, fy, fz, e;
-  int nin;
-  float r2max;  // largest r^2 counted inside ...
-  int jmax;     // ... and its atom (checked exactly when r2max lies in the band)
-};
+// per coordinate).  The loop counts every pair with FP32 r^2 < rc^2 (1 + 2e-6)
+// and keeps the smallest distance of any r^2 from that limit; a lane that saw
+// one near the band (about one in 1500 sub-lists) goes over its list again and
+// takes out the pairs that the 42-bit separations put outside.  The result
+// equals the FP64 test on the full positions except for pairs within ~1e-11
+// of rc.
 
-// The cutoff constants the pair loop keeps in registers; the band's lower
-// edge and rc^2 in 42-bit units are read from the step constants (shared
-// memory) only after the loop, so that they hold no register during it.
-struct MixedCut {
-  float hi;         // rc^2 (1 + 2e-6), units (L / 2^32)^2
-  float inv_lam2;   // (2^32 / L)^2
+// Packed FP32 pairs (one 64-bit register pair; low half first).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ float lo2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ float min3_abs(float a, float b, float c) {
+  float v;
+  asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(v) : "f"(a), "f"(b), "f"(c));
+  return v;
+}
+
+struct PairAcc {
+  f32x2 fx, fy, fz;  // force sums over the even and the odd entries
+  f32x2 e, n;        // ENERGY: pair energies, pairs counted inside
+  float tmin;        // smallest |r^2 - rc^2 (1 + 2e-6)| met
 };
 
 // 42-bit minimum-image separation of one coordinate: top 32 bits (hj, hi) and
@@ -158,59 +198,65 @@ __device__ __forceinline__ bool inside_cutoff_42(uint4 pi, uint4 pj, double x42)
   return fma(dx, dx, fma(dy, dy, dz * dz)) < x42;
 }
 
-// The pair force on i from j: fs * d with fs = s^4 (24 - 48 s^3), s = 1/r^2
-// (sigma units), d = (dx, dy, dz); energy 4 s^3 (s^3 - 1).
-template <bool ENERGY>
-__device__ __forceinline__ void mixed_pair_add(float r2, float dx, float dy, float dz,
-                                               float inv_lam2, float sign, MixedAcc& a) {
-  const float s = rcp_approx(r2) * inv_lam2;
-  const float s3 = s * s * s;
-  const float fs = sign * (s * s3) * fmaf(-48.0f, s3, 24.0f);
-  a.fx = fmaf(fs, dx, a.fx);
-  a.fy = fmaf(fs, dy, a.fy);
-  a.fz = fmaf(fs, dz, a.fz);
+// q and s^4 (1 + q) of two pairs from their r^2, s = -(2^k / r^2), q = c3 s^3.
+// The scale 2^k (cs, exact) keeps the powers in range; the one rounded constant
+// c3 enters once (a rounded scale would enter seven times).
+__device__ __forceinline__ void lj2(f32x2 r2, f32x2 cs, f32x2 c3, f32x2& q, f32x2& fs) {
+  const f32x2 s = mul2(pack2(rcp_approx(lo2(r2)), rcp_approx(hi2(r2))), cs);
+  const f32x2 s2 = mul2(s, s);
+  q = mul2(mul2(s2, s), c3);
+  const f32x2 s4 = mul2(s2, s2);
+  fs = fma2(q, s4, s4);
+}
+
+__device__ __forceinline__ f32x2 len2(f32x2 dx, f32x2 dy, f32x2 dz) {
+  return fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+}
+
+// Atom i against two list entries j, k.  TAIL: only the first `real` of them
+// count (list padding, which may be the atom itself).
+template <bool ENERGY, bool TAIL>
+__device__ __forceinline__ void mixed_pair2(const Hi3& pi, uint4 pj, uint4 pk, f32x2 cs, f32x2 c3, f32x2 nhi,
+                                            int real, PairAcc& a) {
+  const f32x2 dx = pack2((float)(int)(pj.x - pi.x), (float)(int)(pk.x - pi.x));
+  const f32x2 dy = pack2((float)(int)(pj.y - pi.y), (float)(int)(pk.y - pi.y));
+  const f32x2 dz = pack2((float)(int)(pj.z - pi.z), (float)(int)(pk.z - pi.z));
+  const f32x2 r2 = len2(dx, dy, dz);
+  const f32x2 t = add2(r2, nhi);  // negative: inside (the sign is exact)
+  a.tmin = min3_abs(lo2(t), hi2(t), a.tmin);
+  const f32x2 m = pack2(__saturatef(lo2(t) * -1e30f), __saturatef(hi2(t) * -1e30f));
+  f32x2 q, fs;
+  lj2(r2, cs, c3, q, fs);
+  fs = mul2(fs, m);
+  if (TAIL) fs = pack2(real > 0 ? lo2(fs) : 0.0f, real > 1 ? hi2(fs) : 0.0f);
+  a.fx = fma2(fs, dx, a.fx);
+  a.fy = fma2(fs, dy, a.fy);
+  a.fz = fma2(fs, dz, a.fz);
   if (ENERGY) {
-    a.e = fmaf(sign * s3, fmaf(4.0f, s3, -4.0f), a.e);
-    a.nin += (int)sign;
-  }
-}
-
-// Every pair with FP32 r^2 < cut.hi is counted inside; a.r2max and a.jmax
-// remember the largest such r^2 and its atom.  The caller then checks that
-// pair exactly when it lies in the band (mixed_cut_fix).
-template <bool ENERGY, bool MAYBE_SELF>
-__device__ __forceinline__ void mixed_pair(uint4 pi, uint4 pj, int j, const MixedCut& cut,
-                                           MixedAcc& a) {
-  const float dx = (float)(int)(pj.x - pi.x);
-  const float dy = (float)(int)(pj.y - pi.y);
-  const float dz = (float)(int)(pj.z - pi.z);
-  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  // r2 == 0 only for the atom itself (sub-list padding, last block only);
-  // distinct atoms at distance 0 are reported by the list build
-  if (r2 < cut.hi && (!MAYBE_SELF || r2 > 0.0f)) {
-    if (r2 > a.r2max) {
-      a.r2max = r2;
-      a.jmax = j;
+    f32x2 e = mul2(fma2(q, q, add2(q, q)), m), n = m;
+    if (TAIL) {
+      e = pack2(real > 0 ? lo2(e) : 0.0f, real > 1 ? hi2(e) : 0.0f);
+      n = pack2(real > 0 ? lo2(n) : 0.0f, real > 1 ? hi2(n) : 0.0f);
     }
-    mixed_pair_add<ENERGY>(r2, dx, dy, dz, cut.inv_lam2, 1.0f, a);
+    a.e = add2(a.e, e);
+    a.n = add2(a.n, n);
   }
 }
 
-// After the sub-list: if the largest r^2 counted lies in the band and the
-// 42-bit separations put that pair outside rc, take its contribution out
-// again.  (A second band pair in one sub-list -- about one sub-list in 1e8 --
-// stays counted as the FP32 test decided.)
+// Takes one pair's contribution out again.
 template <bool ENERGY>
-__device__ __forceinline__ void mixed_cut_fix(const uint4* pos, int i, const StepConst& K,
-                                              MixedAcc& a) {
-  if (a.r2max > K.rc2u_lo) {
-    const uint4 pi = pos[i], pj = pos[a.jmax];
-    if (!inside_cutoff_42(pi, pj, K.rc2x)) {
-      const float dx = (float)(int)(pj.x - pi.x);
-      const float dy = (float)(int)(pj.y - pi.y);
-      const float dz = (float)(int)(pj.z - pi.z);
-      mixed_pair_add<ENERGY>(a.r2max, dx, dy, dz, K.inv_lam2, -1.0f, a);
-    }
+__device__ __forceinline__ void mixed_pair_remove(float dx, float dy, float dz, float r2,
+                                                  const StepConst& K, PairAcc& a) {
+  f32x2 q, fs;
+  lj2(pack2(r2, r2), pack2(K.cs, K.cs), pack2(K.c3, K.c3), q, fs);
+  const f32x2 m = pack2(-1.0f, 0.0f);
+  fs = mul2(fs, m);
+  a.fx = fma2(fs, pack2(dx, dx), a.fx);
+  a.fy = fma2(fs, pack2(dy, dy), a.fy);
+  a.fz = fma2(fs, pack2(dz, dz), a.fz);
+  if (ENERGY) {
+    a.e = fma2(fma2(q, q, add2(q, q)), m, a.e);
+    a.n = add2(a.n, m);
   }
 }
 
@@ -700,50 +746,77 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
   return finish_sublist(cnt, blk, out, i, zeros > (self ? 1 : 0), cap_sub, overflow);
 }
 
-// Mixed-precision sub-list loop of lane (i, q); see mixed_pair.
-// Sub-lists are padded with the atom's own index up to a whole block of four;
-// only the last block can hold padding, so only it tests for the atom itself.
-// ENERGY: also sum the pair energies (needed only when U is reported).
+// Mixed-precision forces of atom i from this lane's sub-list; see mixed_pair2.
+// ENERGY: also the pair energies (only when U is reported).
 template <bool ENERGY>
-__device__ __forceinline__ MixedAcc mixed_sublist_forces(int i, const uint4* __restrict__ pos,
-                                                         const uint16_t* __restrict__ nb,
-                                                         uint32_t col, uint32_t ncols, int cnt,
-                                                         const StepConst& K) {
-  MixedAcc a{0.f, 0.f, 0.f, 0.f, 0, 0.f, 0};
-  const MixedCut cut{K.rc2u_hi, K.inv_lam2};
-  const uint4 pi = pos[i];
-  const size_t stride4 = (size_t)ncols * 4;
-  const uint16_t* base = nb + (size_t)col * 4;
+__device__ __forceinline__ PairAcc mixed_sublist_forces(Hi3 pi, const uint4* pos,
+                                                        const uint16_t* __restrict__ nb,
+                                                        uint32_t col, uint32_t ncols, int cnt,
+                                                        const StepConst& K) {
+  PairAcc a{0ull, 0ull, 0ull, 0ull, 0ull, 3.0e38f};
+  const f32x2 cs = pack2(K.cs, K.cs), c3 = pack2(K.c3, K.c3);
+  const f32x2 nhi = pack2(-K.rc2u_hi, -K.rc2u_hi);
+  const uint2* list = reinterpret_cast<const uint2*>(nb) + col;
   const int nblk = (cnt + 3) >> 2;
   const int nfull = cnt >> 2;
-  uint2 w = nblk > 0 ? *reinterpret_cast<const uint2*>(base) : make_uint2(0u, 0u);
+  uint2 w = nblk > 0 ? *list : make_uint2(0u, 0u);
   for (int kb = 0; kb < nfull; ++kb) {
     // the next block of indices is requested before this block is used
-    const uint2 wn = kb + 1 < nblk ? *reinterpret_cast<const uint2*>(base + (size_t)(kb + 1) * stride4) : w;
-    const int j0 = w.x & 0xFFFFu, j1 = w.x >> 16, j2 = w.y & 0xFFFFu, j3 = w.y >> 16;
-    const uint4 p0 = pos[j0];
-    const uint4 p1 = pos[j1];
-    const uint4 p2 = pos[j2];
-    const uint4 p3 = pos[j3];
-    mixed_pair<ENERGY, false>(pi, p0, j0, cut, a);
-    mixed_pair<ENERGY, false>(pi, p1, j1, cut, a);
-    mixed_pair<ENERGY, false>(pi, p2, j2, cut, a);
-    mixed_pair<ENERGY, false>(pi, p3, j3, cut, a);
+    list += ncols;
+    const uint2 wn = kb + 1 < nblk ? *list : w;
+    const uint4 p0 = pos[w.x & 0xFFFFu], p1 = pos[w.x >> 16];
+    const uint4 p2 = pos[w.y & 0xFFFFu], p3 = pos[w.y >> 16];
+    mixed_pair2<ENERGY, false>(pi, p0, p1, cs, c3, nhi, 2, a);
+    mixed_pair2<ENERGY, false>(pi, p2, p3, cs, c3, nhi, 2, a);
     w = wn;
   }
-  if (nblk > nfull) {
-    const int j0 = w.x & 0xFFFFu, j1 = w.x >> 16, j2 = w.y & 0xFFFFu, j3 = w.y >> 16;
-    const uint4 p0 = pos[j0];
-    const uint4 p1 = pos[j1];
-    const uint4 p2 = pos[j2];
-    const uint4 p3 = pos[j3];
-    mixed_pair<ENERGY, true>(pi, p0, j0, cut, a);
-    mixed_pair<ENERGY, true>(pi, p1, j1, cut, a);
-    mixed_pair<ENERGY, true>(pi, p2, j2, cut, a);
-    mixed_pair<ENERGY, true>(pi, p3, j3, cut, a);
+  if (nblk > nfull) {  // the last block, in part padding
+    const int left = cnt & 3;
+    const uint4 p0 = pos[w.x & 0xFFFFu], p1 = pos[w.x >> 16];
+    mixed_pair2<ENERGY, true>(pi, p0, p1, cs, c3, nhi, left, a);
+    const uint4 p2 = pos[w.y & 0xFFFFu];
+    mixed_pair2<ENERGY, true>(pi, p2, p2, cs, c3, nhi, left - 2, a);
   }
-  mixed_cut_fix<ENERGY>(pos, i, K, a);
   return a;
+}
+
+// Whole warps: the lanes that met an r^2 near the band (`near`) take out again
+// what the 42-bit separations put outside rc.  The warp goes over such a lane's
+// list together (one lane alone would hold up its CTA for as long as the whole
+// pair loop takes, in most steps of a large replica).
+template <bool ENERGY>
+__device__ __forceinline__ void mixed_cut_fix(bool near, int i, const uint4* pos,
+                                              const uint16_t* __restrict__ nb, uint32_t col,
+                                              uint32_t ncols, int cnt, const StepConst& K,
+                                              PairAcc& a) {
+  const int lane = threadIdx.x & 31;
+  for (uint32_t todo = __ballot_sync(0xffffffffu, near); todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1;
+    const int n = __shfl_sync(0xffffffffu, cnt, src);
+    const uint32_t c = __shfl_sync(0xffffffffu, col, src);
+    const uint4 pi = pos[__shfl_sync(0xffffffffu, i, src)];
+    for (int k0 = 0; k0 < n; k0 += 32) {
+      const int k = k0 + lane;
+      int j = 0;
+      bool band = false;
+      if (k < n) {
+        j = nb[((size_t)(k >> 2) * ncols + c) * 4 + (k & 3)];
+        const uint4 pj = pos[j];
+        const float dx = (float)(int)(pj.x - pi.x), dy = (float)(int)(pj.y - pi.y),
+                    dz = (float)(int)(pj.z - pi.z);
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        band = r2 > K.rc2u_lo && r2 < K.rc2u_hi && !inside_cutoff_42(pi, pj, K.rc2x);
+      }
+      for (uint32_t hit = __ballot_sync(0xffffffffu, band); hit; hit &= hit - 1) {
+        const uint4 pj = pos[__shfl_sync(0xffffffffu, j, __ffs(hit) - 1)];
+        if (lane == src) {
+          const float dx = (float)(int)(pj.x - pi.x), dy = (float)(int)(pj.y - pi.y),
+                      dz = (float)(int)(pj.z - pi.z);
+          mixed_pair_remove<ENERGY>(dx, dy, dz, fmaf(dx, dx, fmaf(dy, dy, dz * dz)), K, a);
+        }
+      }
+    }
+  }
 }
 
 __device__ __forceinline__ void fp64_sublist_forces(Pos64 pi, const Pos64* pos, const uint16_t* nb,
