@@ -39,12 +39,15 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   // replica constants live in shared memory, not in registers
   __shared__ EnsHdr E;
   __shared__ StepConst K;
-  __shared__ double alpha_sh, kp_sh;
+  __shared__ double alpha_sh;
   __shared__ float eps_sh;
   __shared__ int st_sh;
   // free-running exchange: the result handed to the cluster (velocity scale,
   // new T, status), the replica's current T and the launch's first attempt
   // number (thread 0), own steps since the last pattern (warp 0 of CTA 0)
+  __shared__ double sqT_sh;  // FP64 path: sqrt(T)
+  __shared__ Fp64Const fc_sh;
+  __shared__ double fu_sh;   // FP64 path: force unit of the pair sums
   __shared__ double xs_sh, xT_sh, xl_sh, xu_sh, Tcur_sh;
   __shared__ long long A0_sh;
   __shared__ int xst_sh, since_sh, fold0_sh;
@@ -62,6 +65,12 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
     A0_sh = S.attempt[rd.ens];
     since_sh = 0;
     fold0_sh = 0;
+    if (FP64) {
+      sqT_sh = sqrt(Tcur_sh);
+      const double i2 = 1.0 / (K.lam64 * K.lam64);  // (2^64 / L)^2
+      fc_sh = Fp64Const{-2.0 * i2 * i2 * i2, K.rc2 * i2, K.uc};
+      fu_sh = 24.0 * i2 * i2 * i2 * (i2 * K.lam64);
+    }
   }
   const int T = blockDim.x, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5, nw = (T + 31) >> 5;
@@ -239,6 +248,8 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
                              sm.act + warp * row_list_bytes(N), K.rl2u, nb, mycol, ncols,
                              S.raw + rd.nbr_off, (uint32_t)(i * P + q), (uint32_t)(N * P), cap_sub,
                              &overflow);
+      // the FP64 pair loop's notes overlie the screening vectors
+      if (FP64 && P >= 4) __syncthreads();
     }
     if (own) {
 #pragma unroll
@@ -256,26 +267,28 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
     long long iu = 0, ik = 0;  // mixed: fixed-point partial sums
     double du = 0.0, dk = 0.0; // FP64 path
     if (FP64) {
-      double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
-      if (own)
-        fp64_sublist_forces(pos64[i], pos64, nb, mycol, ncols, cnt, K.lam64, K.rc2, K.uc, fx, fy,
-                            fz, e);
+      uint16_t* buf = reinterpret_cast<uint16_t*>(sm.hk);
+      const Fp64Acc a = energy ? fp64_sublist_forces<true, P>(pos64, i, own, nb, mycol, ncols, cnt,
+                                                              buf, K, fc_sh)
+                               : fp64_sublist_forces<false, P>(pos64, i, own, nb, mycol, ncols, cnt,
+                                                               buf, K, fc_sh);
+      double fx = a.fx, fy = a.fy, fz = a.fz, e = a.e;
       fx = group_sum<P>(fx);
       fy = group_sum<P>(fy);
       fz = group_sum<P>(fz);
-      e = group_sum<P>(e);
+      if (energy) e = group_sum<P>(e);  // uniform flag
       if (own) {
         if (q == 0) du = e;
 #pragma unroll
         for (int j = 0; j < ND; ++j) {
           const int d = q + j * P;
           if (d >= 3) continue;
-          f[j] = K.lamv * (d == 0 ? fx : (d == 1 ? fy : fz));
+          f[j] = K.lamv * fu_sh * (d == 0 ? fx : (d == 1 ? fy : fz));
           if (kick) v[j] += K.hdt * f[j];
           dk += v[j] * v[j];
         }
       }
-      du = warp_sum(du);
+      if (energy) du = warp_sum(du);
       dk = warp_sum(dk);
     } else {
       PairAcc a{0ull, 0ull, 0ull, 0ull, 0ull, 3.0e38f};
@@ -329,19 +342,19 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       }
     }
   };
-  // Every warp sums the published partials in the same fixed order and reads
-  // the status bits of every CTA.  FP64 path: sums of FP64 values.  Mixed
+  // A warp sums the published partials in a fixed order and reads the status
+  // bits of every CTA.  FP64 path: sums of FP64 values.  Mixed
   // path: exact 64-bit integer sums of the fixed-point partials.
-  auto totals_fp64 = [&](double& su, double& sk, int& st) {
+  auto totals_fp64 = [&](double& su, double& sk, int& st, bool energy) {
     const long long* uk = reinterpret_cast<const long long*>(sm.slot_uk);
     su = 0.0;
     sk = 0.0;
-    for (int idx = lane; idx < C * kMaxWarps; idx += 32)
-      if (idx % kMaxWarps < nw) {
-        su += __longlong_as_double(uk[idx * 2 + 0]);
-        sk += __longlong_as_double(uk[idx * 2 + 1]);
-      }
-    su = warp_sum(su);
+    for (int idx = lane; idx < C * nw; idx += 32) {
+      const int at = (idx / nw) * kMaxWarps + idx % nw;
+      su += __longlong_as_double(uk[at * 2 + 0]);
+      sk += __longlong_as_double(uk[at * 2 + 1]);
+    }
+    if (energy) su = warp_sum(su);
     sk = warp_sum(sk);
     st = 0;
     for (int rk = 0; rk < C; ++rk) st |= sm.slot_st[rk];
@@ -386,7 +399,7 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
     csync();
     if (FP64) {
       double su, sk;
-      totals_fp64(su, sk, status);
+      totals_fp64(su, sk, status, true);
       const double U0 = 0.5 * su * K.lamv, K0 = 0.5 * sk;
       if (!isfinite(U0) || !isfinite(K0)) status |= kStNumeric;
       if (tid == 0) {
@@ -491,34 +504,35 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
     // the step ends on a materialised step boundary (velocities at full step)
     const bool bnd = last || xchg;
     if (FP64) {
-      double su, sk;
-      totals_fp64(su, sk, st);
-      st &= ~(int)kStXchg;
-      if (z.bad) st |= kStRngCap;
-      const double Un = 0.5 * su * K.lamv, Kn = 0.5 * sk;
-      // one lane forms the FP64 factor and K'; the CTA reads both after the
-      // barrier, so every thread takes the same decisions below
-      if (tid == 0) {
+      // warp 0 forms the totals, the FP64 factor and K'; the CTA reads them after
+      // the barrier, so every thread takes the same decisions below
+      if (warp == 0) {
+        double su, sk;
+        totals_fp64(su, sk, st, energy);
+        st &= ~(int)kStXchg;
+        if (z.bad) st |= kStRngCap;
+        const double Un = 0.5 * su * K.lamv, Kn = 0.5 * sk;
         double alpha = 1.0, kp = Kn;
-        if (thermo) alpha = svr_alpha(Kn, K.kbar, K.nf, K.c_th, z.r1, z.s, &kp);
-        alpha_sh = alpha;
-        kp_sh = kp;
+        if (thermo)
+          alpha = svr_alpha_step(Kn, K.af1 * Tcur_sh, K.bf1 * sqT_sh, K.c_th, z.r1, z.s, &kp);
+        if (!isfinite(alpha) || (energy && !isfinite(Un)) || !isfinite(kp)) st |= kStNumeric;
+        if (lane == 0) {
+          alpha_sh = alpha;
+          st_sh = st;
+          if (energy) U_sh = Un;
+          K_sh = kp;
+          econs_sh += Kn - kp;
+        }
       }
       __syncthreads();
       const double alpha = alpha_sh;
-      const double Kp = kp_sh;
-      if (!isfinite(alpha) || !isfinite(Un) || !isfinite(Kp)) st |= kStNumeric;
+      st = st_sh;
       if (own) {
 #pragma unroll
         for (int j = 0; j < ND; ++j) {
           v[j] *= alpha;
           if (!bnd) v[j] += K.hdt * f[j];  // first half kick of the next step
         }
-      }
-      if (tid == 0) {
-        U_sh = Un;
-        K_sh = Kp;
-        econs_sh += Kn - Kp;
       }
     } else {
       // warp 0 forms the integer totals and alpha - 1 (FP32); the block reads
@@ -662,6 +676,7 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
         if (Tn != Tcur_sh) {
           set_thermo_target(K, Tn);
           Tcur_sh = Tn;
+          if (FP64) sqT_sh = sqrt(Tn);
         }
         if (new_lam) set_potential_scale(K, ln);
         since_sh = 0;

@@ -340,7 +340,12 @@ LaunchCfg wide_cfg(const LaunchCfg& k) {
 }
 
 // Default launch shape: enough CTAs per replica to cover the SMs in about one
-// wave, then as many threads per atom as fit in one CTA (at most 4).
+// wave, then as many threads per atom as fit in one CTA: at most 4, or 8 on the
+// FP64 path, whose pair loop deals its FP64 turns out evenly over an atom's
+// lanes and wants warps to hide its other latencies (8 x 256 atoms: 41 against
+// 45 thousand clocks a step, 20 x 864: 111 against 132).  (Clusters of 16 CTAs
+// for a few FP64 replicas gain nothing: the FP64 units are shared by the two
+// SMs of a pair.)
 LaunchCfg default_cfg(const re_ctx* c, const Scope& sc) {
   LaunchCfg k{};
   const int sms = sm_count();
@@ -355,7 +360,7 @@ LaunchCfg default_cfg(const re_ctx* c, const Scope& sc) {
   }
   int p = c->opt.atom_threads;
   if (p <= 0) {
-    p = 4;
+    p = c->opt.precision == RE_PREC_FP64 ? 8 : 4;
     while (p > 1 && threads_for(sc.max_n, cl, p) > 1024) p /= 2;
   }
   k.cluster = cl;

@@ -138,6 +138,20 @@ __device__ inline double svr_alpha(double K, double Kbar, int nf, double c, doub
   return alpha;
 }
 
+// svr_alpha for the batched kernel's step, where one warp forms it while the
+// others wait: with the constants a = (1 - c) Kbar / Nf and b = 2 sqrt(c a) the
+// new energy is c K + a (R1^2 + S) + b R1 sqrt(K), 1/K and sqrt(K) come from
+// one reciprocal root, and the sign test R1 + sqrt(c K / a) < 0 needs no root:
+// two root-like operations in a row instead of four divisions and three roots.
+__device__ inline double svr_alpha_step(double K, double a, double b, double c, double r1,
+                                        double s, double* Knew) {
+  const double y = rsqrt(K);
+  const double kp = fma(c, K, fma(a, fma(r1, r1, s), b * r1 * (K * y)));
+  const double alpha = sqrt(kp) * y;
+  *Knew = kp;
+  return r1 < 0.0 && a * r1 * r1 > c * K ? -alpha : alpha;
+}
+
 // ------------------------------------------------------------- fixed point
 // A coordinate x in the periodic box [0, L) is stored as q = x/L * 2^64
 // (uint64, wrapping).  The difference of two such words read as a signed

@@ -299,7 +299,10 @@ __host__ __device__ inline size_t batched_layout(int max_n, int threads, bool fp
   const size_t o_pos = take((size_t)max_n * (fp64 ? 32 : 16), 32);  // at the base: fixed offset
   const size_t o_nbs = take(list_elems * 2, 16);
   const size_t rows = ((size_t)max_n + 31) / 32;  // of 32 atoms
-  const size_t o_hk = take(rows * 512, 128);
+  // the screening vectors of a list build, or the FP64 pair loop's notes (32 a
+  // thread; with P >= 4 threads an atom, at most 2048 atoms in 8 CTAs)
+  const size_t hk_bytes = rows * 512, notes = fp64 && max_n <= 2048 ? (size_t)threads * 64 : 0;
+  const size_t o_hk = take(hk_bytes > notes ? hk_bytes : notes, 128);
   const size_t o_bx = take(rows * sizeof(uint2), 8);
   const size_t o_ar = take((size_t)kMaxWarps * row_list_bytes(max_n), 8);
   const size_t o_noise = take((size_t)kNoiseChunk * 2 * kSvrStepBytes, 16);
@@ -819,30 +822,137 @@ __device__ __forceinline__ void mixed_cut_fix(bool near, int i, const uint4* pos
   }
 }
 
-__device__ __forceinline__ void fp64_sublist_forces(Pos64 pi, const Pos64* pos, const uint16_t* nb,
-                                                    uint32_t col, uint32_t ncols, int cnt,
-                                                    double lam64, double rc2, double uc,
-                                                    double& fx, double& fy, double& fz,
-                                                    double& e) {
-  fx = fy = fz = e = 0.0;
-  const size_t stride = ncols;
-  for (int k = 0; k < cnt; ++k) {
-    const int j = nb[((size_t)(k >> 2) * stride + col) * 4 + (k & 3)];
-    const Pos64 pj = pos[j];
-    const double dx = (double)(long long)(pj.x - pi.x) * lam64;
-    const double dy = (double)(long long)(pj.y - pi.y) * lam64;
-    const double dz = (double)(long long)(pj.z - pi.z) * lam64;
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    if (r2 < rc2) {
-      const double s = 1.0 / r2;
-      const double s3 = s * s * s;
-      const double fs = 48.0 * s3 * s3 * s - 24.0 * s3 * s;
-      fx -= fs * dx;
-      fy -= fs * dy;
-      fz -= fs * dz;
-      e += 4.0 * (s3 * s3 - s3) - uc;
+// v 2^-64 as a double, v a positive normal float, by its bits (the conversion
+// instruction runs on the FP64 unit).
+__device__ __forceinline__ double float_to_double_2m64(float v) {
+  const uint32_t u = __float_as_uint(v);
+  return __hiloint2double((int)((u >> 3) + 0x34000000u), (int)(u << 29));
+}
+
+// FP64 force of one pair, separation d (units of L / 2^64), hi the FP32 r^2 of
+// its top words: 17 FP64 operations.  1/r^2 starts from the FP32 value x0 with
+// one third-order step x = x0 (1 + e + e^2), e = 1 - r^2 x0 (the partial sum
+// of the geometric series of 1 / (1 - e)), |e| < 1e-6.  All stay in units of
+// the separation: s = 1/r^2 is about 1e-37 and s^7 about 1e-260, in range.
+// edge: decided on the FP64 r^2.
+struct Fp64Acc {
+  double fx, fy, fz, e;  // sums of 24 s^4 (1 - 2 s^3) d and of the pair energies
+};
+struct Fp64Const {
+  double m2, rc2, uc;  // -2 s3 factor (2^64 / L)^6, rc^2 in these units, shift
+};
+template <bool ENERGY>
+__device__ __forceinline__ void fp64_pair(const Pos64& pi, const Pos64& pj, const Hi3& hi, bool edge,
+                                          const Fp64Const& c, Fp64Acc& a) {
+  const double dx = (double)(long long)(pj.x - pi.x), dy = (double)(long long)(pj.y - pi.y),
+               dz = (double)(long long)(pj.z - pi.z);
+  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+  if (edge && !(r2 < c.rc2)) return;
+  const double x0 = float_to_double_2m64(
+      rcp_approx(sep2_hi(hi, Hi3{(uint32_t)(pj.x >> 32), (uint32_t)(pj.y >> 32), (uint32_t)(pj.z >> 32)})));
+  const double er = fma(-r2, x0, 1.0);
+  const double s = fma(x0, fma(er, er, er), x0);
+  const double s2 = s * s, s3 = s2 * s;
+  const double q = fma(c.m2, s3, 1.0);
+  const double fs = (s2 * s2) * q;
+  a.fx = fma(fs, dx, a.fx);
+  a.fy = fma(fs, dy, a.fy);
+  a.fz = fma(fs, dz, a.fz);
+  if (ENERGY) {
+    const double t = c.m2 * s3;  // -2 s^3 in sigma units: 4 (s^6 - s^3) = t (t + 2)
+    a.e += fma(t, t + 2.0, -c.uc);
+  }
+}
+
+// FP64 pair forces of atom i from its sub-lists, whole warps.  The FP64 unit
+// (1.7 operations per clock and SM, whatever the active lanes) bounds this
+// loop, so everything else is kept off it, and its turns are kept full: FP32
+// distances on the top 32 bits first pick the entries inside the cutoff (55 of
+// 95 at the default skin), 32 entries of a lane at a time; only those take an
+// FP64 turn.  With P >= 4 lanes of an atom the hits of all of them are then
+// dealt out evenly (buf: 32 noted entries a thread in shared memory), since
+// one lane's 14 +- 3 hits would make the fullest of 32 lanes need 21 to 24
+// turns; with fewer lanes each goes through its own hits (a bit mask), 28 +- 4
+// or 55 +- 5 of them.  Entries within 2e-6 of rc^2 are decided on the FP64
+// r^2.
+template <bool ENERGY, int P>
+__device__ __forceinline__ Fp64Acc fp64_sublist_forces(const Pos64* pos, int i, bool own,
+                                                       const uint16_t* __restrict__ nb, uint32_t col,
+                                                       uint32_t ncols, int cnt, uint16_t* buf,
+                                                       const StepConst& K, const Fp64Const& c) {
+  Fp64Acc a{0.0, 0.0, 0.0, 0.0};
+  const Pos64 pi = pos[own ? i : 0];
+  const Hi3 hi{(uint32_t)(pi.x >> 32), (uint32_t)(pi.y >> 32), (uint32_t)(pi.z >> 32)};
+  if (!own) cnt = 0;
+  const int nmax = __reduce_max_sync(0xffffffffu, cnt);
+  auto hi_of = [&](int j) {
+    return Hi3{(uint32_t)(pos[j].x >> 32), (uint32_t)(pos[j].y >> 32), (uint32_t)(pos[j].z >> 32)};
+  };
+  for (int k0 = 0; k0 < nmax; k0 += 32) {
+    uint32_t m = 0, band = 0;  // P < 4: bit k is entry k0 + k
+    int n = 0;                 // P >= 4: noted entries
+    uint16_t* mine = P >= 4 ? buf + threadIdx.x * 32 : nullptr;
+    const uint2* list = reinterpret_cast<const uint2*>(nb) + (size_t)(k0 >> 2) * ncols + col;
+    uint2 wn = make_uint2(0u, 0u);
+    if (k0 < cnt) wn = *list;
+    for (int b = 0; b < 32 && k0 + b < cnt; b += 4) {
+      const uint2 w = wn;
+      list += ncols;
+      if (k0 + b + 4 < cnt) wn = *list;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t j = ((k < 2 ? w.x : w.y) >> (16 * (k & 1))) & 0xFFFFu;
+        const float r2 = sep2_hi(hi, hi_of((int)j));
+        const bool hit = k0 + b + k < cnt && r2 < K.rc2u_hi, edge = r2 > K.rc2u_lo;
+        if (P >= 4) {
+          if (hit) mine[n++] = (uint16_t)(j | (edge ? 0x8000u : 0u));
+        } else if (hit) {
+          m |= 1u << (b + k);
+          if (edge) band |= 1u << (b + k);
+        }
+      }
+    }
+    if (P >= 4) {
+      // hit number r of the atom, r = q, q + P, ...: note r - first[l] of lane l
+      const int lane = threadIdx.x & 31, g0 = lane & ~(P - 1);
+      int first[P + 1];
+      first[0] = 0;
+#pragma unroll
+      for (int l = 0; l < P; ++l) first[l + 1] = first[l] + __shfl_sync(0xffffffffu, n, g0 + l);
+      __syncwarp();
+      const uint16_t* group = buf + (threadIdx.x & ~(P - 1)) * 32;
+      for (int r = lane & (P - 1); __any_sync(0xffffffffu, r < first[P]); r += P) {
+        if (r < first[P]) {
+          int at = r;
+#pragma unroll
+          for (int l = 1; l < P; ++l)
+            if (r >= first[l]) at = r - first[l] + 32 * l;
+          const uint32_t j = group[at];
+          fp64_pair<ENERGY>(pi, pos[j & 0x7FFFu], hi, j >> 15, c, a);
+        }
+      }
+      __syncwarp();
+    } else {
+      auto entry = [&](int k) {
+        return (int)nb[((size_t)((k0 + k) >> 2) * ncols + col) * 4 + (k & 3)];
+      };
+      int k = __ffs(m) - 1;
+      int j = k >= 0 ? entry(k) : 0;
+      while (__any_sync(0xffffffffu, m != 0u)) {
+        if (m != 0u) {
+          const int jc = j;
+          const bool edge = (band >> k) & 1u;
+          m &= m - 1;
+          if (m != 0u) {  // the next turn's entry is read one turn ahead
+            k = __ffs(m) - 1;
+            j = entry(k);
+          }
+          fp64_pair<ENERGY>(pi, pos[jc], hi, edge, c, a);
+        }
+      }
     }
   }
+  return a;
 }
 
 template <int P>
