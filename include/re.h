@@ -358,11 +358,13 @@ int re_exchange_device_h(int R, const double *T, const double *lam, const double
 /* Truncated LJ forces and potential energy of N atoms in a cubic periodic box
  * of side L with cutoff rc (Example section): x device array of 3N doubles
  * (AoS), f device array of 3N doubles, U device pointer to one double.
- * Pairs are found with the same cell binning and neighbour-list kernels as
- * the MD path (list radius rc + skin, skin = 0.5).  precision: RE_PREC_FP64
- * or RE_PREC_MIXED.  Scratch (cells, lists) is allocated with cudaMalloc and
- * freed before return; the call synchronises `stream`.  Requires 2 <= N <=
- * 65535 and rc + 0.5 < L/2. */
+ * precision: RE_PREC_FP64 or RE_PREC_MIXED, with the pair arithmetic of the MD
+ * path; the replica sizes and, within rc + 0.5 of an atom, the neighbours that
+ * its default lists hold are the limits (RE_EINVAL, RE_EOVERFLOW beyond).
+ * Scratch comes from a memory pool of the library's own, stream-ordered, and
+ * goes back before return; the call synchronises `stream`.  Calls from several
+ * threads and streams do not affect one another.  Requires 2 <= N <= 65535 and
+ * rc + 0.5 < L/2. */
 int re_lj_forces_device(int N, double L, double rc, int shift, int precision, const double *x,
                         double *f, double *U, void *stream);
 
@@ -371,8 +373,8 @@ int re_lj_forces_device(int N, double L, double rc, int shift, int precision, co
  * another framework's memory pool or under a fixed memory budget, plug-ins
  * that may not touch the allocator).  The paper has no counterpart: this is a
  * deployment variant.  Scratch lives in one fixed device array of about
- * 2.6 MB that every device loading the library keeps until the process exits.
- * Limits: 2 <= N <= 4096 atoms, at most 256 neighbour-list entries per atom
+ * 140 KB that every device loading the library keeps until the process exits.
+ * Limits: 2 <= N <= 4096 atoms, at most 256 neighbours within rc + 0.5 per atom
  * (RE_EOVERFLOW beyond), rc + 0.5 < L/2.  Arguments as re_lj_forces_device
  * (device pointers, caller-owned).  The first call on a device looks up the
  * array's device address and caches it: make that first call before any

@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -2210,6 +2211,41 @@ int re_exchange_device_h(int R, const double* T, const double* lam, const double
   return RE_OK;
 }
 
+namespace {
+
+// The memory pool of re_lj_forces_device on the current device: stream-ordered,
+// so calls from any threads and streams share it; it keeps at most 64 MB between
+// calls (the driver's pools grow by 32 MB; keeping less than that, every call
+// maps memory anew, 220 us) and returns the rest.  The some 45 allocations of a
+// context took half a millisecond a call and more.
+cudaError_t scratch_pool(cudaMemPool_t* out) {
+  static std::mutex mu;
+  static cudaMemPool_t pools[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+    uint64_t keep = 64ull << 20;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    pools[dev] = p;
+  }
+  *out = pools[dev];
+  return cudaSuccess;
+}
+
+}  // namespace
+
 int re_lj_forces_device(int N, double L, double rc, int shift, int precision, const double* x,
                         double* f, double* U, void* stream) {
   g_create_error.clear();
@@ -2219,43 +2255,52 @@ int re_lj_forces_device(int N, double L, double rc, int shift, int precision, co
     return fail(nullptr, RE_EINVAL, "need rc + 0.5 < L/2");
   if (precision != RE_PREC_FP64 && precision != RE_PREC_MIXED)
     return fail(nullptr, RE_EINVAL, "unknown precision");
-  // A one-replica context without lattice set-up: import x, prologue, export f.
-  re_ctx* c = new re_ctx();
-  re_default_opts(&c->opt);
-  c->opt.precision = precision;
-  c->opt.shift_energy = shift;
-  c->stream = static_cast<cudaStream_t>(stream);
-  cudaGetDevice(&c->device);
-  Ensemble e{N, 1, L, rc, {1.0}, 0};
-  int rcode = build_context(c, {e}, nullptr);
-  auto bail = [&](int code) {
-    g_create_error = c->err;
-    re_destroy(c);
-    return code;
-  };
-  if (rcode) return bail(rcode);
-  const double one = 1.0;
-  int32_t zero = 0;
-  cudaError_t ce;
-  if ((ce = cudaMemcpyAsync(c->s.T, &one, 8, cudaMemcpyHostToDevice, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.vx, 0, 8 * (size_t)N, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.vy, 0, 8 * (size_t)N, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.vz, 0, 8 * (size_t)N, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.econs, 0, 8, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.step, 0, 8, c->stream)) ||
-      (ce = cudaMemsetAsync(c->s.nreb, 0, 8, c->stream)) ||
-      (ce = cudaMemcpyAsync(c->s.status, &zero, 4, cudaMemcpyHostToDevice, c->stream)))
-    return bail(cuda_fail(c, ce, "set-up"));
-  ce = re::launch_import_state(c->s, c->d_ens, c->d_rep, 1, x, nullptr, c->stream);
-  if (ce != cudaSuccess) return bail(cuda_fail(c, ce, "import"));
-  rcode = refresh(c);
-  if (rcode == RE_OK) rcode = status_check(c);
-  if (rcode) return bail(rcode);
-  ce = re::launch_export_state(c->s, c->d_ens, c->d_rep, 1, nullptr, nullptr, f, c->stream);
-  if (ce == cudaSuccess) ce = cudaMemcpyAsync(U, c->s.U, 8, cudaMemcpyDeviceToDevice, c->stream);
-  if (ce == cudaSuccess) ce = cudaStreamSynchronize(c->stream);
-  if (ce != cudaSuccess) return bail(cuda_fail(c, ce, "export"));
-  re_destroy(c);
+  // the sizes that a one-replica context of this precision takes
+  re_ctx c;
+  re_default_opts(&c.opt);
+  c.opt.precision = precision;
+  EnsDev e{};
+  e.N = N;
+  e.R = 1;
+  e.L = L;
+  e.rc = rc;
+  e.skin = c.opt.skin;
+  e.rlist = rc + c.opt.skin;
+  e.dt = c.opt.dt;
+  e.tau = c.opt.tau_T;
+  e.shift = shift ? 1 : 0;
+  set_capacity(e, 0);
+  finish_ens(e);
+  c.ens.push_back(e);
+  c.n_rep = c.max_r = 1;
+  c.max_n = N;
+  apply_cells(&c, 0);
+  const LaunchCfg cfg = default_cfg(&c);
+  if (check_cfg(&c, cfg) != RE_OK) return fail(nullptr, RE_EINVAL, "%s", c.err.c_str());
+  // the neighbours that lists of up to four threads per atom hold
+  int p = 4;
+  while (p > 1 && threads_for(N, cfg.cluster, p) > 1024) p /= 2;
+  const int cap = p * e.capsub[p == 1 ? 0 : (p == 2 ? 1 : 2)];
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaMemPool_t pool = nullptr;
+  cudaError_t ce = scratch_pool(&pool);
+  if (ce != cudaSuccess) return cuda_fail(nullptr, ce, "scratch pool");
+  void* scratch = nullptr;
+  ce = cudaMallocFromPoolAsync(&scratch, re::direct_scratch_bytes(N), pool, st);
+  if (ce != cudaSuccess) return cuda_fail(nullptr, ce, "scratch");
+  int32_t* d_status = nullptr;
+  int32_t status = 0;
+  ce = re::launch_lj_direct(scratch, N, e.kc, precision == RE_PREC_MIXED, cap, sm_count(), x, f, U,
+                            &d_status, st);
+  if (ce == cudaSuccess)
+    ce = cudaMemcpyAsync(&status, d_status, sizeof status, cudaMemcpyDeviceToHost, st);
+  const cudaError_t cf = cudaFreeAsync(scratch, st);
+  const cudaError_t cs = cudaStreamSynchronize(st);
+  for (cudaError_t k : {ce, cf, cs})
+    if (k != cudaSuccess) return cuda_fail(nullptr, k, "forces");
+  if (status & re::kStOverflow)
+    return fail(nullptr, RE_EOVERFLOW, "neighbour list capacity exceeded (%d per atom)", cap);
+  if (status) return fail(nullptr, RE_ENUMERIC, "non-finite energy (overlapping atoms?)");
   return RE_OK;
 }
 

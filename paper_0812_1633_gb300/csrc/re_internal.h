@@ -252,6 +252,19 @@ cudaError_t launch_identity_perm(const StateDev& s, const EnsDev* d_ens, const R
 cudaError_t launch_spatial_sort(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                                 int n_rep, int max_n, int max_ncell, int64_t n_atoms,
                                 cudaStream_t st);
+// Forces and energy of one configuration (re_forces.cu): positions, partial sums
+// and words of a call in one scratch area of direct_scratch_bytes(N) bytes,
+// 16-byte aligned; N <= 32767.  cap: neighbours within the list radius of K
+// that an atom may have (beyond: kStOverflow in *status, a device word).
+struct DirectScratch {
+  uint4 *hi, *lo;  // N each: top and low 32 bits of the fixed-point positions
+  double* part;    // energy of each CTA
+  int32_t* words;  // CTAs done, status bits
+};
+size_t direct_scratch_bytes(int N);
+cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixed, int cap, int sms,
+                             const double* x, double* f, double* U, int32_t** status,
+                             cudaStream_t st);
 cudaError_t launch_exchange_raw(int R, const double* T, const double* lam, const double* U,
                                 uint64_t seed, int64_t attempt, int parity_mode, int distance,
                                 double* T_out, double* lam_out, int32_t* partner,
