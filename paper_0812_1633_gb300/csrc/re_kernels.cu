@@ -304,60 +304,16 @@ __global__ void plain_thermo(StateDev S, const EnsDev* __restrict__ ens,
 }
 
 // ------------------------------------------------------------------ exchange
-// Sorted order of R distinct positive keys (ascending; ties, which the API
-// excludes, by index): a bitonic sort of (key, index) pairs over the next
-// power of two m >= R in shared memory -- keyd and order hold m entries, the
-// first R keys set by the caller, the padding sorts last.  Positive doubles
-// order like their IEEE bit patterns read as 64-bit integers, so the
-// comparisons run on the integer units instead of the (1/64-rate) FP64 unit.
-__device__ void sort_keys(double* keyd, int* order, int R) {
-  long long* key = reinterpret_cast<long long*>(keyd);
-  int m = 1;
-  while (m < R) m <<= 1;
-  for (int t = threadIdx.x; t < m; t += blockDim.x) {
-    if (t >= R) key[t] = LLONG_MAX;
-    order[t] = t;
-  }
-  __syncthreads();
-  for (int k = 2; k <= m; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int t = threadIdx.x; t < m; t += blockDim.x) {
-        const int u = t ^ j;
-        if (u > t) {
-          const bool up = (t & k) == 0;
-          const long long ka = key[t], kb = key[u];
-          const int ia = order[t], ib = order[u];
-          if ((ka > kb || (ka == kb && ia > ib)) == up) {
-            key[t] = kb;
-            key[u] = ka;
-            order[t] = ib;
-            order[u] = ia;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// shared memory of sort_keys for R keys
-__host__ __device__ inline size_t sort_keys_bytes(int R) {
-  size_t m = 1;
-  while (m < (size_t)R) m <<= 1;
-  return m * (sizeof(double) + sizeof(int));
-}
-
 // Ladders up to this size are ordered by one CTA counting ranks (every thread
 // scans all keys, broadcast reads, no barriers); longer ones by
 // exchange_cluster_kernel.
 constexpr int kRankSortMax = 256;
 
-// shared memory of exchange_kernel for R replicas: sort_keys' area (12 bytes
-// per key slot: not a multiple of 8 for a one-replica ladder), then, from the
-// next 16-byte boundary, per replica the quotients lam/T and U/lam, the
-// exchange uniform, T and lam
+// shared memory of exchange_kernel for R replicas: keys and order (12 bytes per
+// replica), then, from the next 16-byte boundary, per replica the quotients
+// lam/T and U/lam, the exchange uniform, T and lam
 __host__ __device__ inline size_t exchange_dbl_offset(int R) {
-  return (sort_keys_bytes(R) + 15) / 16 * 16;
+  return ((size_t)R * 12 + 15) / 16 * 16;
 }
 __host__ __device__ inline size_t exchange_smem_bytes(int R) {
   return exchange_dbl_offset(R) + (size_t)R * 5 * sizeof(double);
@@ -384,10 +340,8 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
   const int parity_mode = ens[blockIdx.x].parity_mode;
   const uint64_t seed = ens[blockIdx.x].seed;
   const int64_t attempt = S.attempt[blockIdx.x];
-  int m = 1;
-  while (m < R) m <<= 1;
   double* key = reinterpret_cast<double*>(sh);
-  int* order = reinterpret_cast<int*>(key + m);
+  int* order = reinterpret_cast<int*>(key + R);
   double* qt = reinterpret_cast<double*>(sh + exchange_dbl_offset(R));  // lam / T
   double* qu = qt + R;                                               // U / lam
   double* uni = qu + R;                                              // uniform of id a
@@ -406,22 +360,18 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
     if (acc_out) acc_out[base + a] = 0;
   }
   __syncthreads();
-  if (R <= kRankSortMax) {
-    // positive doubles order like their bit patterns; ties (excluded by the
-    // API) by index, as sort_keys
-    const long long* ki = reinterpret_cast<const long long*>(key);
-    for (int a = threadIdx.x; a < R; a += blockDim.x) {
-      const long long ka = ki[a];
-      int rank = 0;
+  // positive doubles order like their bit patterns; ties (excluded by the API)
+  // by index
+  const long long* ki = reinterpret_cast<const long long*>(key);
+  for (int a = threadIdx.x; a < R; a += blockDim.x) {
+    const long long ka = ki[a];
+    int rank = 0;
 #pragma unroll 8
-      for (int b = 0; b < R; ++b) {
-        const long long kb = ki[b];
-        rank += (kb < ka) | ((kb == ka) & (b < a));
-      }
-      order[rank] = a;
+    for (int b = 0; b < R; ++b) {
+      const long long kb = ki[b];
+      rank += (kb < ka) | ((kb == ka) & (b < a));
     }
-  } else {
-    sort_keys(key, order, R);
+    order[rank] = a;
   }
   __syncthreads();
   const int p = pair_offset(parity_mode, seed, attempt);
@@ -608,57 +558,86 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
   if (cr == 0 && tid == 0) S.attempt[e] = attempt + 1;
 }
 
-__global__ void exchange_raw_kernel(int R, const double* __restrict__ T,
-                                    const double* __restrict__ lam,
-                                    const double* __restrict__ U, uint64_t seed, int64_t attempt,
-                                    int mode, int distance, double* T_out, double* lam_out,
-                                    int32_t* partner, uint8_t* acc, double* vscale,
-                                    double* uscale) {
+// The stateless attempt, on a cluster of C CTAs (one for up to 128 replicas):
+// every CTA reads the whole ladder's keys and ranks its slice of the replicas
+// by counting, as exchange_cluster_kernel, and hands the order to every CTA;
+// then one thread per replica (not per pair) finds its partner by its own
+// position and forms its own results: of the chain of FP64 divisions, roots
+// and the exponential (several hundred clocks each) only D and exp(D) follow
+// one another, the rest runs beside them.  Bound by that chain and the
+// launch: 5.9 us for 64 replicas (one thread a pair and a bitonic sort: 7.8),
+// 16.6 for 1000 with lam (46.9 on one CTA).  The decision is metropolis(): both
+// members of a pair evaluate it on the same values in the same order.
+__global__ void __launch_bounds__(512) exchange_raw_kernel(
+    int R, const double* __restrict__ T, const double* __restrict__ lam,
+    const double* __restrict__ U, uint64_t seed, int64_t attempt, int mode, int distance,
+    double* T_out, double* lam_out, int32_t* partner, uint8_t* acc, double* vscale,
+    double* uscale) {
   extern __shared__ __align__(16) unsigned char sh[];
-  int m = 1;
-  while (m < R) m <<= 1;
-  double* key = reinterpret_cast<double*>(sh);
-  int* order = reinterpret_cast<int*>(key + m);
-  for (int a = threadIdx.x; a < R; a += blockDim.x) {
-    const double l = lam ? lam[a] : 1.0;
-    key[a] = T[a] / l;
-    T_out[a] = T[a];
-    if (lam_out) lam_out[a] = l;
-    partner[a] = -1;
-    acc[a] = 0;
-    vscale[a] = 1.0;
-    if (uscale) uscale[a] = 1.0;
-  }
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+  long long* key = reinterpret_cast<long long*>(sh);  // R: T/lam as bit patterns
+  int* order = reinterpret_cast<int*>(key + R);       // R: replica at each ladder position
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int a = tid; a < R; a += nt) key[a] = __double_as_longlong(lam ? T[a] / lam[a] : T[a]);
   __syncthreads();
-  sort_keys(key, order, R);
-  __syncthreads();
-  const int p = pair_offset(mode, seed, attempt);
-  const int d = max(1, distance);
-  for (int q = threadIdx.x; q < R; q += blockDim.x) {
-    const int qb = ladder_partner(q, R, p, d);
-    if (qb <= q) continue;
-    const int a = order[q], b = order[qb];
-    const double Ta = T[a], Tb = T[b];
-    const double la = lam ? lam[a] : 1.0, lb = lam ? lam[b] : 1.0;
-    const bool ok = metropolis(Ta, Tb, la, lb, U[a], U[b], seed, min(a, b), attempt);
-    partner[a] = b;
-    partner[b] = a;
-    if (ok) {
-      acc[a] = acc[b] = 1;
-      vscale[a] = sqrt(Tb / Ta);
-      vscale[b] = sqrt(Ta / Tb);
-      T_out[a] = Tb;
-      T_out[b] = Ta;
-      if (lam_out) {
-        lam_out[a] = lb;
-        lam_out[b] = la;
-      }
-      if (uscale) {
-        uscale[a] = lb / la;
-        uscale[b] = la / lb;
+  const int per = (R + C - 1) / C;
+  const int a0 = min(R, cr * per), a1 = min(R, a0 + per);
+  // G threads (consecutive lanes, G a power of two <= 32) per replica
+  int G = 1;
+  while (G < 32 && G * 2 * per <= nt) G *= 2;
+  for (int t0 = 0; t0 < per * G; t0 += nt) {
+    const int t = t0 + tid;
+    const int a = a0 + t / G, part = t % G;
+    const bool mine = t < per * G && a < a1;
+    int rank = 0;
+    if (mine) {
+      const long long ka = key[a];
+#pragma unroll 4
+      for (int b = part; b < R; b += G) {
+        const long long kb = key[b];
+        rank += (kb < ka) | ((kb == ka) & (b < a));
       }
     }
+    for (int o = G / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (mine && part == 0)
+      for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(order + rank, rk) = a;
   }
+  if (C > 1)
+    cl.sync();
+  else
+    __syncthreads();
+  const int p = pair_offset(mode, seed, attempt);
+  const int d = max(1, distance);
+  for (int q = a0 + tid; q < a1; q += nt) {
+    const int m = order[q], qb = ladder_partner(q, R, p, d);
+    const double Tm = T[m], lm = lam ? lam[m] : 1.0;
+    double Tn = Tm, ln = lm, vs = 1.0, us = 1.0;
+    int other = -1;
+    bool ok = false;
+    if (qb >= 0) {
+      other = order[qb];
+      const double To = T[other], lo = lam ? lam[other] : 1.0;
+      const bool first = q < qb;  // metropolis() takes the pair in ladder order
+      const double Um = U[m], Uo = U[other];
+      const double root = sqrt(To / Tm), ratio = lam ? lo / lm : 1.0;
+      ok = metropolis(first ? Tm : To, first ? To : Tm, first ? lm : lo, first ? lo : lm,
+                      first ? Um : Uo, first ? Uo : Um, seed, min(m, other), attempt);
+      if (ok) {
+        Tn = To;
+        ln = lo;
+        vs = root;
+        us = ratio;
+      }
+    }
+    T_out[m] = Tn;
+    if (lam_out) lam_out[m] = ln;
+    partner[m] = other;
+    acc[m] = ok ? 1 : 0;
+    vscale[m] = vs;
+    if (uscale) uscale[m] = us;
+  }
+  if (C > 1) cl.sync();  // no CTA leaves while another may still write its order
 }
 
 // Exchange results decided elsewhere (a ladder sharded over several
@@ -1148,16 +1127,28 @@ cudaError_t launch_exchange_raw(int R, const double* T, const double* lam, const
                                 double* T_out, double* lam_out, int32_t* partner,
                                 uint8_t* accepted, double* vscale, double* uscale,
                                 cudaStream_t st) {
-  const size_t smem = sort_keys_bytes(R);
-  const int threads = R >= 512 ? 512 : ((R + 31) / 32) * 32;
+  // about 128 replicas per CTA, at most 8 CTAs; one CTA needs no cluster launch
+  const int C = std::min(8, (R + 127) / 128);
+  const size_t smem = (size_t)R * (sizeof(long long) + sizeof(int));
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(exchange_raw_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  exchange_raw_kernel<<<1, threads, smem, st>>>(R, T, lam, U, seed, attempt, parity_mode, distance,
-                                               T_out, lam_out, partner, accepted, vscale, uscale);
-  return cudaGetLastError();
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)C);
+  lc.blockDim = dim3(512);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&lc, exchange_raw_kernel, R, T, lam, U, seed, attempt, parity_mode,
+                            distance, T_out, lam_out, partner, accepted, vscale, uscale);
 }
 
 }  // namespace re
