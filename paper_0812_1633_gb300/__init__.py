@@ -297,8 +297,8 @@ class Context:
         return lam
 
     def get_state(self):
-        x = np.zeros((self.n_atoms, 3))
-        v = np.zeros((self.n_atoms, 3))
+        x = np.empty((self.n_atoms, 3))
+        v = np.empty((self.n_atoms, 3))
         _check(lib().re_get_state(self._h, _p(x, C.c_double), _p(v, C.c_double)), self._h)
         return x, v
 

@@ -2,6 +2,8 @@
 // per replica) and its launch helpers, instantiated per precision and mode in
 // the re_batched_*.cu translation units so that they compile in parallel.
 #pragma once
+#include <mutex>
+
 #include "re_md.cuh"
 
 namespace re {
@@ -742,6 +744,45 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
 
 }  // namespace
 
+// What the driver was last told about one kernel: shared memory and carve-out.
+// Launches of contexts, threads and devices that alternate between shapes set
+// them again; a repeated launch asks nothing (four driver calls, 5 us, of the
+// 20 that a synchronised cycle's launches took).
+struct PreparedLaunch {
+  std::mutex mu;
+  int dev = -1, threads = 0;
+  size_t smem = 0;
+};
+
+inline cudaError_t prepare_batched(const void* fn, int threads, size_t smem, PreparedLaunch* p) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(p->mu);
+  if (p->dev == dev && p->threads == threads && p->smem == smem) return cudaSuccess;
+  p->dev = -1;
+  cudaFuncAttributes fa{};
+  e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess) return e;
+  if (fa.sharedSizeBytes > kBatchedStaticSmem) return cudaErrorInvalidConfiguration;
+  // the limit stays at the largest any launch may ask for: lowering it here
+  // could undercut another thread's launch
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(232448 - fa.sharedSizeBytes));
+  if (e != cudaSuccess) return e;
+  // the rest of the SM's 256 KB serves as L1 (lists in global memory, state)
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
+  per_sm = std::max(1, per_sm);
+  const int carve = (int)std::min<size_t>(100, (per_sm * (smem + 1024) * 100 + 232447) / 232448);
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+  if (e != cudaSuccess) return e;
+  p->dev = dev;
+  p->threads = threads;
+  p->smem = smem;
+  return cudaSuccess;
+}
+
 template <bool FP64, int P, bool LSM, int MODE, int MAXT>
 cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                                    const int* d_work, int n_work, const int32_t* d_budget,
@@ -750,18 +791,8 @@ cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDe
                                    const FreeDev* fr) {
   const size_t smem = batched_smem_bytes(max_n, cfg.threads, FP64, list_elems);
   auto fn = md_batched_kernel<FP64, P, LSM, MODE, MAXT>;
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaFuncGetAttributes(&fa, fn);
-  if (e != cudaSuccess) return e;
-  if (fa.sharedSizeBytes > kBatchedStaticSmem) return cudaErrorInvalidConfiguration;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  // the rest of the SM's 256 KB serves as L1 (lists in global memory, state)
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, cfg.threads, smem);
-  per_sm = std::max(1, per_sm);
-  const int carve = (int)std::min<size_t>(100, (per_sm * (smem + 1024) * 100 + 232447) / 232448);
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
+  static PreparedLaunch prepared;  // of this instantiation
+  cudaError_t e = prepare_batched(reinterpret_cast<const void*>(fn), cfg.threads, smem, &prepared);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)(n_work * cfg.cluster));
@@ -779,7 +810,11 @@ cudaError_t launch_batched_t(const StateDev& s, const EnsDev* d_ens, const RepDe
   FreeDev f{};
   if (fr) f = *fr;
   e = cudaLaunchKernelEx(&lc, fn, s, d_ens, d_rep, d_work, d_budget, dims, f);
-  if (e != cudaSuccess) cudaGetLastError();  // a refused launch leaves no error behind
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // a refused launch leaves no error behind
+    std::lock_guard<std::mutex> lock(prepared.mu);
+    prepared.dev = -1;   // ask the driver again at the next one
+  }
   return e;
 }
 
@@ -787,8 +822,10 @@ template <bool FP64, int P, bool LSM, int MAXT>
 int max_active_clusters_t(const LaunchCfg& cfg, int max_n, size_t list_elems) {
   const size_t smem = batched_smem_bytes(max_n, cfg.threads, FP64, list_elems);
   auto fn = md_batched_kernel<FP64, P, LSM, 2, MAXT>;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(232448 - fa.sharedSizeBytes)) != cudaSuccess)
     return 0;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)cfg.cluster);

@@ -393,11 +393,10 @@ int allocate(re_ctx* c) {
       (rc = dalloc(c, &s.rx, A)) || (rc = dalloc(c, &s.ry, A)) || (rc = dalloc(c, &s.rz, A)) ||
       (rc = dalloc(c, &s.ncnt, 8 * A)) || (rc = dalloc(c, &s.nbr, (size_t)c->n_nbr)) ||
       (c->opt.path == RE_PATH_BATCHED && (rc = dalloc(c, &s.raw, (size_t)c->n_nbr))) ||
-      (rc = dalloc(c, &s.T, R)) || (rc = dalloc(c, &s.U, R)) || (rc = dalloc(c, &s.K, R)) ||
-      (rc = dalloc(c, &s.econs, R)) || (rc = dalloc(c, &s.vscale, R)) ||
+      (rc = dalloc(c, &s.T, R)) || (rc = dalloc(c, &s.U, 4 * R)) || (rc = dalloc(c, &s.vscale, R)) ||
       (rc = dalloc(c, &s.lam, R)) || (rc = dalloc(c, &s.fscale, R)) ||
       (rc = dalloc(c, &s.step, R)) || (rc = dalloc(c, &s.nreb, R)) ||
-      (rc = dalloc(c, &s.status, R)) || (rc = dalloc(c, &s.valid, R)) ||
+      (rc = dalloc(c, &s.valid, R)) ||
       (rc = dalloc(c, &s.attempt, E)) || (rc = dalloc(c, &s.pair_att, (size_t)c->n_pairs)) ||
       (rc = dalloc(c, &s.pair_acc, (size_t)c->n_pairs)) ||
       (rc = dalloc(c, &s.red, R * 1024)) || (rc = dalloc(c, &s.dmax, R)) ||
@@ -409,9 +408,15 @@ int allocate(re_ctx* c) {
       (rc = dalloc(c, &c->d_work_id, R)) || (rc = dalloc(c, &c->d_zero, R)) ||
       (rc = dalloc(c, &c->d_work_ord, R)) ||
       (rc = dalloc(c, &c->d_budget, R)) ||
-      (rc = dalloc(c, &c->d_budget_nx, R)) || (rc = dalloc(c, &c->d_partner, R)) ||
-      (rc = dalloc(c, &c->d_acc, R)) || (rc = dalloc(c, &c->d_io, 3 * A)))
+      (rc = dalloc(c, &c->d_budget_nx, R)) || (rc = dalloc(c, &c->d_partner, 2 * R)) ||
+      (rc = dalloc(c, &c->d_io, 3 * A)))
     return rc;
+  // what is read back together lies together, laid out like h_out: the energies
+  // and the status words, the partners and the decisions
+  s.K = s.U + R;
+  s.econs = s.U + 2 * R;
+  s.status = reinterpret_cast<int32_t*>(s.U + 3 * R);
+  c->d_acc = reinterpret_cast<uint8_t*>(c->d_partner + R);
   RE_CUDA(c, cudaMemsetAsync(s.nbr, 0, sizeof(uint16_t) * (size_t)c->n_nbr, c->stream), "memset");
   RE_CUDA(c, cudaMemsetAsync(c->d_zero, 0, sizeof(int32_t) * R, c->stream), "memset");
   RE_CUDA(c, cudaMemsetAsync(s.ncnt, 0, sizeof(int32_t) * 8 * A, c->stream), "memset");
@@ -569,7 +574,7 @@ int launch_class(re_ctx* c, int e, const int32_t* d_budget, cudaStream_t st, boo
   }
   cudaError_t err = re::launch_batched(c->s, c->d_ens, c->d_rep, work, c->ens[e].R, d_budget,
                                        c->opt.precision == RE_PREC_FP64, k, sc.max_n,
-                                       list_elems_for(c, k, sc), 0, st, nullptr);
+                                       list_elems_for(c, k, sc), 0, st, nullptr, uneven);
   if (err != cudaSuccess) return cuda_fail(c, err, "batched MD launch (ensemble class)");
   return RE_OK;
 }
@@ -670,7 +675,7 @@ int launch_advance(re_ctx* c, const int32_t* d_budget, const int32_t* h_budget,
       if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch (wide class)");
       e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work2, nn, d_budget, fp64, c->cfg,
                              c->max_n, list_elems_for(c, c->cfg), 0, c->stream,
-                             nullptr);
+                             nullptr, uneven);
       if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
       RE_CUDA(c, cudaEventRecord(c->ev_join, c->side), "join");
       RE_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0), "join");
@@ -686,7 +691,7 @@ int launch_advance(re_ctx* c, const int32_t* d_budget, const int32_t* h_budget,
     cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, order ? c->d_work_ord : c->d_work,
                                        c->n_rep, d_budget, fp64, k, c->max_n,
                                        budgets ? list_elems_for(c, k) : 0, async_nx,
-                                       c->stream, fr);
+                                       c->stream, fr, budgets && uneven);
     if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch");
     return RE_OK;
   }
@@ -1293,13 +1298,9 @@ int re_exchange(re_ctx* c, int32_t* partner_out, uint8_t* accepted_out) {
                                       c->d_acc, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "exchange launch");
   if (!partner_out && !accepted_out) return RE_OK;
-  // through the pinned read-back area: truly asynchronous copies, one wait
-  if (partner_out)
-    RE_CUDA(c, cudaMemcpyAsync(out_partner(c), c->d_partner, sizeof(int32_t) * c->n_rep,
-                               cudaMemcpyDeviceToHost, c->stream), "read partners");
-  if (accepted_out)
-    RE_CUDA(c, cudaMemcpyAsync(out_acc(c), c->d_acc, c->n_rep, cudaMemcpyDeviceToHost, c->stream),
-            "read accepted");
+  // through the pinned read-back area: one asynchronous copy, one wait
+  RE_CUDA(c, cudaMemcpyAsync(out_partner(c), c->d_partner, 5 * (size_t)c->n_rep,
+                             cudaMemcpyDeviceToHost, c->stream), "read partners and decisions");
   RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
   if (partner_out) std::memcpy(partner_out, out_partner(c), sizeof(int32_t) * c->n_rep);
   if (accepted_out) std::memcpy(accepted_out, out_acc(c), c->n_rep);
@@ -1583,14 +1584,10 @@ int re_run_record(re_ctx* c, int n_cycles, const int32_t* steps, int use_graph, 
 int re_energies(re_ctx* c, double* U, double* K, double* H) {
   ApiRange range_("re_energies");
   if (!c) return fail(nullptr, RE_EINVAL, "context is NULL");
-  // status and energies in one synchronisation (pinned destinations)
+  // energies and status in one copy (pinned destination)
   const size_t R = (size_t)c->n_rep;
-  RE_CUDA(c, cudaMemcpyAsync(out_status(c), c->s.status, 4 * R, cudaMemcpyDeviceToHost, c->stream),
-          "read status");
-  RE_CUDA(c, cudaMemcpyAsync(out_U(c), c->s.U, 8 * R, cudaMemcpyDeviceToHost, c->stream), "read U");
-  RE_CUDA(c, cudaMemcpyAsync(out_K(c), c->s.K, 8 * R, cudaMemcpyDeviceToHost, c->stream), "read K");
-  RE_CUDA(c, cudaMemcpyAsync(out_econs(c), c->s.econs, 8 * R, cudaMemcpyDeviceToHost, c->stream),
-          "read econs");
+  RE_CUDA(c, cudaMemcpyAsync(out_U(c), c->s.U, 28 * R, cudaMemcpyDeviceToHost, c->stream),
+          "read energies");
   RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
   int rc = status_eval(c, out_status(c));
   if (rc) return rc;
@@ -1638,29 +1635,25 @@ int re_lambdas(re_ctx* c, double* lam) {
 
 int re_temps(re_ctx* c, double* T) {
   if (!c || !T) return fail(c, RE_EINVAL, "bad arguments");
+  RE_CUDA(c, cudaMemcpyAsync(out_U(c), c->s.T, sizeof(double) * c->n_rep, cudaMemcpyDeviceToHost,
+                             c->stream), "read T");
   RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
-  RE_CUDA(c, cudaMemcpy(T, c->s.T, sizeof(double) * c->n_rep, cudaMemcpyDeviceToHost), "read T");
+  std::memcpy(T, out_U(c), sizeof(double) * c->n_rep);
   return RE_OK;
 }
 
 int re_get_state(re_ctx* c, double* x, double* v) {
   if (!c) return fail(nullptr, RE_EINVAL, "context is NULL");
   const size_t n3 = 3 * (size_t)c->n_atoms;
-  cudaError_t e = re::launch_apply_vscale(c->s, c->d_rep, c->d_ens, c->n_rep, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "apply velocity factors");
-  if (x) {
-    e = re::launch_export_state(c->s, c->d_ens, c->d_rep, c->n_rep, c->d_io, nullptr, nullptr,
-                                c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "export");
-    RE_CUDA(c, cudaMemcpyAsync(x, c->d_io, 8 * n3, cudaMemcpyDeviceToHost, c->stream), "read x");
-    RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
-  }
-  if (v) {
-    e = re::launch_export_state(c->s, c->d_ens, c->d_rep, c->n_rep, nullptr, c->d_io, nullptr,
-                                c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "export");
-    RE_CUDA(c, cudaMemcpyAsync(v, c->d_io, 8 * n3, cudaMemcpyDeviceToHost, c->stream), "read v");
-  }
+  // both in one launch (v into the re-sort's staging words), pending factors of
+  // an exchange applied to what is read
+  double* dv = reinterpret_cast<double*>(c->s.sbuf);
+  const cudaError_t e = re::launch_export_state(c->s, c->d_ens, c->d_rep, c->n_rep,
+                                                x ? c->d_io : nullptr, v ? dv : nullptr, nullptr,
+                                                c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "export");
+  if (x) RE_CUDA(c, cudaMemcpyAsync(x, c->d_io, 8 * n3, cudaMemcpyDeviceToHost, c->stream), "read x");
+  if (v) RE_CUDA(c, cudaMemcpyAsync(v, dv, 8 * n3, cudaMemcpyDeviceToHost, c->stream), "read v");
   RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
   return RE_OK;
 }
@@ -1861,11 +1854,8 @@ int re_forces(re_ctx* c, double* f) {
   if (!c || !f) return fail(c, RE_EINVAL, "bad arguments");
   int rc = status_check(c);
   if (rc) return rc;
-  // pending velocity and force factors of the last exchange become part of the state
-  cudaError_t e = re::launch_apply_vscale(c->s, c->d_rep, c->d_ens, c->n_rep, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "apply pending factors");
-  e = re::launch_export_state(c->s, c->d_ens, c->d_rep, c->n_rep, nullptr, nullptr, c->d_io,
-                              c->stream);
+  const cudaError_t e = re::launch_export_state(c->s, c->d_ens, c->d_rep, c->n_rep, nullptr, nullptr,
+                                                c->d_io, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "export");
   RE_CUDA(c, cudaMemcpyAsync(f, c->d_io, 8 * 3 * (size_t)c->n_atoms, cudaMemcpyDeviceToHost,
                              c->stream), "read f");

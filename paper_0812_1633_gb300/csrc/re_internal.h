@@ -184,6 +184,7 @@ size_t batched_admission_bytes(int max_n, int max_ncell, int threads, bool fp64)
 // Shared memory the batched kernel declares statically (replica constants and
 // hand-over words), reserved on top of batched_smem_bytes; launches check it.
 constexpr size_t kBatchedStaticSmem = 512;
+// uneven: the budgets differ between replicas (they choose the build only).
 // list_elems > 0: each CTA keeps its atoms' neighbour sub-lists (list_elems
 // uint16 entries) in shared memory during the launch
 // async_nx > 0: master-stop mode (budgets ignored): in every ensemble the
@@ -195,7 +196,8 @@ constexpr size_t kBatchedStaticSmem = 512;
 cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                            const int* d_work, int n_work, const int32_t* d_budget, bool fp64,
                            const LaunchCfg& cfg, int max_n, size_t list_elems,
-                           int async_nx, cudaStream_t st, const FreeDev* fr = nullptr);
+                           int async_nx, cudaStream_t st, const FreeDev* fr = nullptr,
+                           bool uneven = false);
 // Clusters of the batched kernel that can be resident at once with this
 // launch shape (0 when the query fails).
 int batched_max_active_clusters(bool fp64, const LaunchCfg& cfg, int max_n);

@@ -707,10 +707,11 @@ __global__ void export_kernel(StateDev S, const EnsDev* __restrict__ ens,
   const int r = blockIdx.y;
   const RepDev rd = reps[r];
   const EnsDev E = ens[rd.ens];
+  const double vs = S.vscale[r], fs = S.fscale[r];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < E.N; i += gridDim.x * blockDim.x) {
     const int g = rd.atom_off + i;
-    // original order (no permutation array: slots are the original order)
-    const size_t o = (size_t)rd.atom_off + (S.perm ? S.perm[g] : i);
+    // original order
+    const size_t o = (size_t)rd.atom_off + S.perm[g];
     if (x) {
       const uint64_t q[3] = {S.qx[g], S.qy[g], S.qz[g]};
       for (int d = 0; d < 3; ++d) {
@@ -719,16 +720,32 @@ __global__ void export_kernel(StateDev S, const EnsDev* __restrict__ ens,
         x[3 * o + d] = xv;
       }
     }
+    // with the pending factors of an exchange: the words and the rounding of the
+    // next launch's start
     if (v) {
-      v[3 * o + 0] = S.vfix ? vfix_to_double(vfix_get(S.vx, g)) : S.vx[g];
-      v[3 * o + 1] = S.vfix ? vfix_to_double(vfix_get(S.vy, g)) : S.vy[g];
-      v[3 * o + 2] = S.vfix ? vfix_to_double(vfix_get(S.vz, g)) : S.vz[g];
+      const double* vc[3] = {S.vx, S.vy, S.vz};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (S.vfix) {
+          const long long w = vfix_get(vc[d], g);
+          v[3 * o + d] = vfix_to_double(vs == 1.0 ? w : vfix_scale(w, vs));
+        } else {
+          v[3 * o + d] = vc[d][g] * vs;
+        }
+      }
     }
     if (f) {
       // mixed path: F = (dt/2 F) / (dt/2), the half-kick increment scaled back
-      f[3 * o + 0] = S.vfix ? (double)hfix_get(S.fx, g) * E.kc.inv_hdt : S.fx[g];
-      f[3 * o + 1] = S.vfix ? (double)hfix_get(S.fy, g) * E.kc.inv_hdt : S.fy[g];
-      f[3 * o + 2] = S.vfix ? (double)hfix_get(S.fz, g) * E.kc.inv_hdt : S.fz[g];
+      const double* fc[3] = {S.fx, S.fy, S.fz};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (S.vfix) {
+          const float h = hfix_get(fc[d], g);
+          f[3 * o + d] = (double)(fs == 1.0 ? h : hfix_scale(h, fs)) * E.kc.inv_hdt;
+        } else {
+          f[3 * o + d] = fc[d][g] * fs;
+        }
+      }
     }
   }
 }
@@ -956,23 +973,48 @@ cudaError_t launch_attempt_add(const StateDev& s, int n_ens, int n, cudaStream_t
   return cudaGetLastError();
 }
 
+// Which build of the batched kernel: the one with 72 registers a thread (at most
+// kNarrowThreads threads) spills less, the one with 64 lets two CTAs of up to
+// 512 threads share an SM (the register file has 16384 for each quarter of an
+// SM, which takes a quarter of a CTA's warps, rounded up).  The latter where
+// the launch has more CTAs than the former holds at once: 48 x 500 atoms in
+// four-CTA clusters of 512 threads, 10 steps, 134 us against 169.  Not with
+// uneven budgets (uneven): there the launch lasts as long as its longest job,
+// which an SM of its own serves better (the same replicas with budgets of 2 to
+// 18 steps: 413 us against 367 for two cycles).
+static bool narrow_build(const LaunchCfg& cfg, int max_n, bool fp64, size_t list_elems, int n_work,
+                         bool uneven) {
+  if (cfg.threads > kNarrowThreads) return false;
+  if (uneven) return true;
+  const size_t smem = batched_smem_bytes(max_n, cfg.threads, fp64, list_elems) + kBatchedStaticSmem + 1024;
+  const int quarter = ((cfg.threads + 31) / 32 + 3) / 4;
+  auto resident = [&](int regs) {
+    return std::min(16384 / (regs * 32 * quarter), (int)(233472 / smem));
+  };
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int n72 = resident(72);
+  return (long long)n_work * cfg.cluster <= (long long)sms * n72 || resident(64) <= n72;
+}
+
 cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                            const int* d_work, int n_work, const int32_t* d_budget, bool fp64,
                            const LaunchCfg& cfg, int max_n, size_t list_elems,
-                           int async_nx, cudaStream_t st, const FreeDev* fr) {
+                           int async_nx, cudaStream_t st, const FreeDev* fr, bool uneven) {
   if (n_work <= 0) return cudaSuccess;
   const bool lsm = list_elems > 0;
   const int mode = (fr && fr->nx > 0) ? 2 : (async_nx > 0 ? 1 : 0);
   // the two free-running modes keep the lists in global memory
   if (mode != 0 && lsm) return cudaErrorInvalidValue;
-#define RE_LB(F, PP, LS, M)                                                                   \
-  return cfg.threads <= kNarrowThreads                                                         \
-             ? launch_batched_t<F, PP, LS, M, kNarrowThreads>(s, d_ens, d_rep, d_work, n_work, \
-                                                              d_budget, cfg, max_n,            \
-                                                              list_elems, async_nx, st, fr)    \
-             : launch_batched_t<F, PP, LS, M, 1024>(s, d_ens, d_rep, d_work, n_work, d_budget, \
-                                                    cfg, max_n, list_elems,                    \
-                                                    async_nx, st, fr);
+  const bool narrow = mode == 2 ? cfg.threads <= kNarrowThreads
+                                : narrow_build(cfg, max_n, fp64, list_elems, n_work, uneven);
+#define RE_LB(F, PP, LS, M)                                                                      \
+  return narrow ? launch_batched_t<F, PP, LS, M, kNarrowThreads>(s, d_ens, d_rep, d_work, n_work, \
+                                                                 d_budget, cfg, max_n,            \
+                                                                 list_elems, async_nx, st, fr)    \
+                : launch_batched_t<F, PP, LS, M, 1024>(s, d_ens, d_rep, d_work, n_work, d_budget, \
+                                                       cfg, max_n, list_elems, async_nx, st, fr);
 #define RE_LBP(F, LS, M)                           \
   switch (cfg.atom_threads) {                      \
     case 1: RE_LB(F, 1, LS, M)                     \
