@@ -120,6 +120,69 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   uint4* posm = reinterpret_cast<uint4*>(smem_raw);
   Pos64* pos64 = reinterpret_cast<Pos64*>(smem_raw);
 
+  // The CTA's own part of the state, requested before the barrier: the loads
+  // overlap thread 0's set-up.  Per lane in registers (the FP32 velocity of the
+  // mixed path is formed from the fixed-point word when needed, and the
+  // positions at the last list build are kept in shared memory: registers are
+  // the scarce resource of this kernel, which holds the state for a whole
+  // launch)
+  const int N = ens[rd.ens].N;
+  const int per = (N + C - 1) / C;
+  const int i0 = min(N, crank * per), i1 = min(N, i0 + per);
+  const int i = i0 + tid / P;
+  const bool own = i < i1;
+  const int g = rd.atom_off + i;
+  int32_t* ncnt = S.ncnt + (size_t)rd.atom_off * 8;
+  uint64_t xq[ND];
+  double v[ND], f[ND];       // FP64 path
+  long long vq[ND];          // mixed path: velocity, fixed point
+  float hf[ND];              // mixed path: half-kick increment
+  // top 32 bits of the coordinates at the last list build: in shared memory
+  // on the mixed path (3 words per own atom), in registers on the FP64 path
+  // (whose shared memory holds 64-bit positions)
+  uint32_t ref_r[ND];
+  int cnt = 0;
+#pragma unroll
+  for (int j = 0; j < ND; ++j) {
+    const int d = q + j * P;
+    xq[j] = 0;
+    v[j] = f[j] = 0.0;
+    vq[j] = 0;
+    hf[j] = 0.0f;
+    ref_r[j] = 0;
+    if (own && d < 3) {
+      xq[j] = qcomp(S, d)[g];
+      ref_r[j] = rcomp(S, d)[g];
+      if (FP64) {
+        v[j] = vcomp(S, d)[g];
+        f[j] = fcomp(S, d)[g];
+      } else {
+        vq[j] = vfix_get(vcomp(S, d), g);
+        hf[j] = hfix_get(fcomp(S, d), g);
+      }
+    }
+  }
+  if (own) cnt = ncnt[(size_t)i * P + q];
+
+  // The thermostat records of kNoiseChunk steps from step s0 of the launch on.
+  // Every CTA of the cluster makes its own identical copy and every record a
+  // step may read is written whatever the block size: the CTAs of a replica
+  // must take the same decisions (a CTA that left the step loop early would
+  // leave its partners writing into the shared memory of an exited block).
+  auto make_noise = [&](int s0) {
+    SvrStep* dst = reinterpret_cast<SvrStep*>(sm.noise) + ((s0 / kNoiseChunk) & 1) * kNoiseChunk;
+    for (int t = tid; t < kNoiseChunk && s0 + t < B; t += T) {
+      int capped = 0;
+      SvrStep z = svr_step(FP64, 3 * N - 3, ens[rd.ens].seed, (uint64_t)rd.stream,
+                           (uint64_t)(step0 + s0 + t), &capped);
+      z.bad = capped;
+      dst[t] = z;
+    }
+  };
+  // the first ones while the state is on its way (a chain of some 3 thousand
+  // clocks that a one-step launch would wait for at its first barrier)
+  if (ens[rd.ens].tau > 0.0) make_noise(0);
+
   // Every CTA has read the replica's flags before any CTA may change them
   // (the barrier also publishes E and K to the whole CTA).
   cl.sync();
@@ -136,12 +199,6 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       __syncthreads();
   };
 
-  const int N = E.N;
-  const int per = (N + C - 1) / C;
-  const int i0 = min(N, crank * per), i1 = min(N, i0 + per);
-  const int i = i0 + tid / P;
-  const bool own = i < i1;
-  const int g = rd.atom_off + i;
   const int cap_sub = E.capsub[P == 1 ? 0 : (P == 2 ? 1 : (P == 4 ? 2 : 3))];
   uint16_t* nbg = S.nbr + rd.nbr_off;  // global lists: columns i * P + q of N * P
   // lists used by the step loop: in shared memory (columns (i - i0) * P + q of
@@ -149,53 +206,27 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   uint16_t* nb = LSM ? sm.nb_sm : nbg;
   const uint32_t ncols = LSM ? (uint32_t)(per * P) : (uint32_t)(N * P);
   const uint32_t mycol = LSM ? (uint32_t)((i - i0) * P + q) : (uint32_t)(i * P + q);
-  int32_t* ncnt = S.ncnt + (size_t)rd.atom_off * 8;
   const float dtqf = (float)K.dtq;
   const float ucf = (float)K.uc;
   const bool thermo = E.tau > 0.0;  // decided once; no FP64 tests inside the step loop
 
-  // per-lane state in registers (the FP32 velocity of the mixed path is
-  // formed from the fixed-point word when needed, and the positions at the
-  // last list build are kept in shared memory: registers are the scarce
-  // resource of this kernel, which holds the state for a whole launch)
-  uint64_t xq[ND];
-  double v[ND], f[ND];       // FP64 path
-  long long vq[ND];          // mixed path: velocity, fixed point
-  float hf[ND];              // mixed path: half-kick increment
-  // top 32 bits of the coordinates at the last list build: in shared memory
-  // on the mixed path (3 words per own atom), in registers on the FP64 path
-  // (whose shared memory holds 64-bit positions)
-  uint32_t ref_r[ND];
   uint32_t* ref_sm = FP64 ? nullptr : sm.ref + (size_t)(i - i0) * 3;
   auto ref = [&](int j) -> uint32_t& { return FP64 ? ref_r[j] : ref_sm[q + j * P]; };
-  int cnt = 0;
 #pragma unroll
   for (int j = 0; j < ND; ++j) {
-    const int d = q + j * P;
-    xq[j] = 0;
-    v[j] = f[j] = 0.0;
-    vq[j] = 0;
-    hf[j] = 0.0f;
-    ref_r[j] = 0;
-    if (own && d < 3) {
-      xq[j] = qcomp(S, d)[g];
-      ref(j) = rcomp(S, d)[g];
-      if (FP64) {
-        v[j] = vcomp(S, d)[g] * vs0;
-        f[j] = fcomp(S, d)[g] * fs0;
-      } else {
-        // the state is stored in these words: FP64 only for a pending factor
-        const long long vb = vfix_get(vcomp(S, d), g);
-        const float hb = hfix_get(fcomp(S, d), g);
-        vq[j] = vs_one ? vb : vfix_scale(vb, vs0);
-        hf[j] = fs_one ? hb : hfix_scale(hb, fs0);
-      }
+    if (!own || q + j * P >= 3) continue;
+    if (FP64) {
+      v[j] *= vs0;
+      f[j] *= fs0;
+    } else {
+      // the state is stored in these words: scaled only by a pending factor
+      ref(j) = ref_r[j];
+      if (!vs_one) vq[j] = vfix_scale(vq[j], vs0);
+      if (!fs_one) hf[j] = hfix_scale(hf[j], fs0);
     }
   }
   // FP32 copy of velocity word j (mixed path)
   auto vf = [&](int j) { return ll2f_split(vq[j]) * kVelUnit; };
-  if (own) cnt = ncnt[(size_t)i * P + q];
-
   auto hi_of = [&](int a) -> Hi3 {
     if (FP64) {
       const Pos64 p = pos64[a];
@@ -424,21 +455,8 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
 
   int done = 0;
   for (int s = 0; s < B && status == 0 && !(freerun && k_next >= fr.n_att); ++s) {
-    const int64_t n = step0 + s;
     SvrStep* sv = reinterpret_cast<SvrStep*>(sm.noise) + ((s / kNoiseChunk) & 1) * kNoiseChunk;
-    // The thermostat records of the next kNoiseChunk steps.  Every CTA of the
-    // cluster makes its own identical copy and every record a step may read
-    // is written whatever the block size: the CTAs of a replica must take the
-    // same decisions (a CTA that left the step loop early would leave its
-    // partners writing into the shared memory of an exited block).
-    if (thermo && (s % kNoiseChunk) == 0) {
-      for (int t = tid; t < kNoiseChunk && s + t < B; t += T) {
-        int capped = 0;
-        SvrStep z = svr_step(FP64, K, E.seed, (uint64_t)rd.stream, (uint64_t)(n + t), &capped);
-        z.bad = capped;
-        sv[t] = z;
-      }
-    }
+    if (thermo && s > 0 && (s % kNoiseChunk) == 0) make_noise(s);
     // (first half kick of the launch) + drift + displacement since the last rebuild
     float d2 = 0.0f;
     if (own) {

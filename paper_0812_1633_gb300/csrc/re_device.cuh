@@ -295,9 +295,19 @@ __device__ __forceinline__ double vfix_to_double(long long vq) { return (double)
 __device__ __forceinline__ long long vfix_from_double(double v) {
   return __double2ll_rn(v * 0x1.0p48);
 }
-// pending factors: v <- v * vs, the half-kick increment (and the force) <- * fs
+// pending factors: v <- v * vs, the half-kick increment (and the force) <- * fs.
+// vs in [2^-10, 2) is an integer of at most 63 bits times 2^-62, so the product
+// is formed exactly in integers and rounded once; FP64 (which rounds it twice)
+// took three operations of the FP64 unit a word, 5.5 thousand clocks of the
+// launch start of a 1024-atom CTA after an accepted exchange.
 __device__ __forceinline__ long long vfix_scale(long long vq, double vs) {
-  return __double2ll_rn((double)vq * vs);
+  const long long b = __double_as_longlong(vs);
+  const int ex = (int)(b >> 52) - 1023;  // the sign bit of a negative factor: out of range
+  if (ex > 0 || ex < -10) return __double2ll_rn((double)vq * vs);
+  const long long m = ((b & 0xFFFFFFFFFFFFFll) | (1ll << 52)) << (10 + ex);
+  const long long hi = __mul64hi(vq, m);
+  const unsigned long long lo = (unsigned long long)vq * (unsigned long long)m;
+  return (long long)(((unsigned long long)hi << 2) | (lo >> 62)) + (long long)((lo >> 61) & 1);
 }
 __device__ __forceinline__ float hfix_scale(float h, double fs) { return (float)((double)h * fs); }
 

@@ -988,19 +988,19 @@ struct SvrStep {
 };
 static_assert(sizeof(SvrStep) == kSvrStepBytes, "thermostat record size");
 
-__device__ inline SvrStep svr_step(bool fp64, const StepConst& K, uint64_t seed, uint64_t stream,
+__device__ inline SvrStep svr_step(bool fp64, int nf, uint64_t seed, uint64_t stream,
                                    uint64_t n, int* capped) {
   SvrStep t;
   t.bad = 0;
   t.pad = 0;
   if (fp64) {
-    const double2 z = svr_noise(K.nf, seed, stream, n, capped);
+    const double2 z = svr_noise(nf, seed, stream, n, capped);
     t.r1 = z.x;
     t.s = z.y;
     t.r1f = (float)z.x;
     t.sf = (float)z.y;
   } else {
-    const float2 z = svr_noise_f32(K.nf, seed, stream, n, capped);
+    const float2 z = svr_noise_f32(nf, seed, stream, n, capped);
     t.r1 = z.x;
     t.s = z.y;
     t.r1f = z.x;
