@@ -6,8 +6,8 @@
 // dt, stochastic velocity rescaling), run for every replica at once:
 //   md_batched_kernel  one thread-block cluster per replica runs that
 //                      replica's whole step budget: kick, drift, displacement
-//                      test, [cell binning + counting sort + list build], LJ
-//                      forces, kick, thermostat.  Positions of the replica
+//                      test, [list build: candidates screened on the tensor
+//                      cores, exact integer test], LJ forces, kick, thermostat.  Positions of the replica
 //                      live in shared memory of every CTA of the cluster
 //                      (broadcast through distributed shared memory).
 //   plain_*            the same step as a sequence of launches for one
@@ -319,6 +319,32 @@ __host__ __device__ inline size_t exchange_smem_bytes(int R) {
   return exchange_dbl_offset(R) + (size_t)R * 5 * sizeof(double);
 }
 
+// The pairs of ladder_partner() by number: pair k's lower position (its upper one
+// is d above; the pair exists if that is below R), and how many numbers there
+// are.  One thread a pair, not one a position: an FP64 instruction occupies its
+// unit for all 32 lanes of a warp (19 clocks), also for those of upper members.
+__device__ __forceinline__ int ladder_pair_low(int k, int p, int d) {
+  return p * d + k / d * (2 * d) + k % d;
+}
+__device__ __forceinline__ int ladder_pairs(int R, int p, int d) {
+  const long long left = (long long)R - (long long)p * d;
+  return left <= d ? 0 : (int)((left + 2ll * d - 1) / (2ll * d) * d);
+}
+
+// The part of replica a's ladder position that keys b = part, part + G, ... give:
+// those smaller, and equal ones (excluded by the API) of a smaller index.  Two
+// loops, so that one comparison an element decides; unrolled, because a short
+// loop waits for the chain of shared-memory loads, not for their number.
+__device__ __forceinline__ int rank_part(const long long* key, int R, int a, int part, int G) {
+  const long long ka = key[a];
+  int rank = 0, b = part;
+#pragma unroll 8
+  for (; b < a; b += G) rank += key[b] <= ka;
+#pragma unroll 8
+  for (; b < R; b += G) rank += key[b] < ka;
+  return rank;
+}
+
 // One exchange attempt per ensemble (one CTA each; contexts whose longest
 // ladder exceeds kRankSortMax use exchange_cluster_kernel): ladder keys T/lam sorted,
 // pairs (q, q + d) of the ladder (d = 1: sorted neighbours), the Metropolis
@@ -329,7 +355,9 @@ __host__ __device__ inline size_t exchange_smem_bytes(int R) {
 // out for latency: one load phase, every per-replica quotient and uniform
 // computed once and in parallel (the same operations as the pair formula, so
 // the decisions are those of metropolis()), and what an accepted pair
-// changes read before the decision.
+// changes read before the decision.  Attempts back to back: 10.3 us for 200
+// replicas, 12.0 for 256 (12.3 and 14.4 with one lane ranking a replica and a
+// thread a position); 8.2 for 64, the launch, either way.
 // rec (may be null): the cycle's record row, per replica id of all rtot
 // replicas T, U, K and econs after the attempt at rec[0..4 rtot).
 __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int32_t* partner_out,
@@ -363,22 +391,21 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
   // positive doubles order like their bit patterns; ties (excluded by the API)
   // by index
   const long long* ki = reinterpret_cast<const long long*>(key);
-  for (int a = threadIdx.x; a < R; a += blockDim.x) {
-    const long long ka = ki[a];
-    int rank = 0;
-#pragma unroll 8
-    for (int b = 0; b < R; ++b) {
-      const long long kb = ki[b];
-      rank += (kb < ka) | ((kb == ka) & (b < a));
-    }
-    order[rank] = a;
+  int G = 1;  // consecutive lanes per replica
+  while (G < 32 && G * 2 * R <= (int)blockDim.x) G *= 2;
+  for (int t0 = 0; t0 < R * G; t0 += blockDim.x) {
+    const int t = t0 + threadIdx.x, a = t / G, part = t % G;
+    int rank = a < R ? rank_part(ki, R, a, part, G) : 0;
+    for (int o = G / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (a < R && part == 0) order[rank] = a;
   }
   __syncthreads();
   const int p = pair_offset(parity_mode, seed, attempt);
   const int d = max(1, xdist);
-  for (int q = threadIdx.x; q < R; q += blockDim.x) {
-    const int qb = ladder_partner(q, R, p, d);
-    if (qb <= q) continue;  // unpaired, or the upper member of its pair
+  const int np = ladder_pairs(R, p, d);
+  for (int k = threadIdx.x; k < np; k += blockDim.x) {
+    const int q = ladder_pair_low(k, p, d), qb = q + d;
+    if (qb >= R) continue;  // the last block may be short
     const int a = order[q], b = order[qb];
     const int ga = base + a, gb = base + b;
     // everything an accepted exchange changes, requested before the decision
@@ -389,6 +416,7 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
     // metropolis(): D = (lam_a/T_a - lam_b/T_b)(U_a/lam_a - U_b/lam_b), accept
     // iff D >= 0 or r < exp(D), r the uniform of the lower replica id
     const double dd = __dmul_rn(__dsub_rn(qt[a], qt[b]), __dsub_rn(qu[a], qu[b]));
+    const double sa = sqrt(Tb / Ta), sb = sqrt(Ta / Tb);  // beside the decision
     const bool ok = dd >= 0.0 || uni[min(a, b)] < exp(dd);
     if (partner_out) {
       partner_out[ga] = b;
@@ -398,7 +426,6 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
     if (ok) {
       S.pair_acc[pair_off + q] = n_acc + 1;
       if (acc_out) acc_out[ga] = acc_out[gb] = 1;
-      const double sa = sqrt(Tb / Ta), sb = sqrt(Ta / Tb);
       const double Kan = Ka * (sa * sa), Kbn = Kb * (sb * sb);
       S.vscale[ga] = va * sa;
       S.vscale[gb] = vb * sb;
@@ -442,11 +469,13 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
 // ranks its slice of the replicas by counting (G threads per replica, each
 // counting over every G-th key, summed by shuffles), writing each replica's
 // ladder position into the order array of every CTA of the cluster
-// (distributed shared memory); after a cluster barrier each CTA runs the
-// pairs whose lower ladder position lies in its slice, with the arithmetic of
-// exchange_kernel, so the decisions are the same.  A second barrier makes
-// every CTA's updates visible before the record is written and the attempt
-// counted.
+// (distributed shared memory); after a cluster barrier each CTA runs its
+// share of the pairs, with the arithmetic of exchange_kernel, so the decisions
+// are the same.  A second barrier makes every CTA's updates visible before the
+// record is written and the attempt counted.  Bound by the counting and the
+// FP64 chain of a pair.  Attempts back to back, with one comparison an element,
+// unrolled, one thread a pair and the factors beside the decision: 17.1 us for
+// 1024 replicas, 141 for 4000, against 24.6 and 209 with a thread a position.
 __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ ens,
                                         int32_t* partner_out, uint8_t* acc_out, double* rec,
                                         int rtot) {
@@ -480,14 +509,7 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
     const int t = t0 + tid;
     const int a = a0 + t / G, part = t % G;
     const bool mine = t < per * G && a < a1;
-    int rank = 0;
-    if (mine) {
-      const long long ka = key[a];
-      for (int b = part; b < R; b += G) {
-        const long long kb = key[b];
-        rank += (kb < ka) | ((kb == ka) & (b < a));
-      }
-    }
+    int rank = mine ? rank_part(key, R, a, part, G) : 0;
     for (int o = G / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (mine && part == 0)
       for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(order + rank, rk) = a;
@@ -495,9 +517,10 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
   cl.sync();
   const int p = pair_offset(parity_mode, seed, attempt);
   const int d = max(1, xdist);
-  for (int q = a0 + tid; q < a1; q += nt) {
-    const int qb = ladder_partner(q, R, p, d);
-    if (qb <= q) continue;
+  const int np = ladder_pairs(R, p, d), perk = (np + C - 1) / C;
+  for (int k = cr * perk + tid; k < min(np, (cr + 1) * perk); k += nt) {
+    const int q = ladder_pair_low(k, p, d), qb = q + d;
+    if (qb >= R) continue;
     const int a = order[q], b = order[qb];
     const int ga = base + a, gb = base + b;
     const long long n_att = S.pair_att[pair_off + q], n_acc = S.pair_acc[pair_off + q];
@@ -508,9 +531,10 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
     const double qta = __ddiv_rn(la, Ta), qtb = __ddiv_rn(lb, Tb);
     const double qua = la == 1.0 ? Ua : __ddiv_rn(Ua, la), qub = lb == 1.0 ? Ub : __ddiv_rn(Ub, lb);
     const double dd = __dmul_rn(__dsub_rn(qta, qtb), __dsub_rn(qua, qub));
-    bool ok = dd >= 0.0;
-    if (!ok)
-      ok = uniforms(seed, (uint64_t)min(a, b), (uint64_t)attempt, kTagExch, 0ull).u0 < exp(dd);
+    // the factors of an acceptance and the uniform do not wait for the decision
+    const double sa = sqrt(Tb / Ta), sb = sqrt(Ta / Tb);
+    const double u = uniforms(seed, (uint64_t)min(a, b), (uint64_t)attempt, kTagExch, 0ull).u0;
+    const bool ok = dd >= 0.0 || u < exp(dd);
     if (partner_out) {
       partner_out[ga] = b;
       partner_out[gb] = a;
@@ -519,7 +543,6 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
     if (ok) {
       S.pair_acc[pair_off + q] = n_acc + 1;
       if (acc_out) acc_out[ga] = acc_out[gb] = 1;
-      const double sa = sqrt(Tb / Ta), sb = sqrt(Ta / Tb);
       const double Kan = Ka * (sa * sa), Kbn = Kb * (sb * sb);
       S.vscale[ga] = va * sa;
       S.vscale[gb] = vb * sb;
@@ -590,15 +613,7 @@ __global__ void __launch_bounds__(512) exchange_raw_kernel(
     const int t = t0 + tid;
     const int a = a0 + t / G, part = t % G;
     const bool mine = t < per * G && a < a1;
-    int rank = 0;
-    if (mine) {
-      const long long ka = key[a];
-#pragma unroll 4
-      for (int b = part; b < R; b += G) {
-        const long long kb = key[b];
-        rank += (kb < ka) | ((kb == ka) & (b < a));
-      }
-    }
+    int rank = mine ? rank_part(key, R, a, part, G) : 0;
     for (int o = G / 2; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (mine && part == 0)
       for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(order + rank, rk) = a;
@@ -1111,7 +1126,8 @@ cudaError_t launch_exchange(const StateDev& s, const EnsDev* d_ens, int n_ens, i
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const int threads = max_r >= 512 ? 512 : ((max_r + 31) / 32) * 32;
+  // eight lanes rank a replica of up to 64, two one of 256
+  const int threads = std::min(512, ((max_r * 8 + 31) / 32) * 32);
   exchange_kernel<<<n_ens, threads, smem, st>>>(s, d_ens, d_partner, d_acc, d_rec, rtot);
   return cudaGetLastError();
 }
