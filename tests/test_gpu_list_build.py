@@ -89,3 +89,24 @@ def test_pairs_at_the_cutoff(re, P, prec):
     ctx.set_state(x)
     check_forces(ctx, N, L, 1, prec)
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("P,cluster", [(4, 4), (2, 2)])
+def test_result_does_not_depend_on_the_register_build(re, P, cluster, prec):
+    """More clusters than fit at once take the build with fewer registers; the
+    same replicas in a smaller context take the other one: equal bit for bit,
+    also with uneven budgets (which keep the larger build)."""
+    N = 500
+    L = inputs.box_length(N)
+    temps = [1.0 + 0.01 * k for k in range(160)]
+    state = []
+    for R in (160, 12):
+        ctx = re.Context(N, L, 2.5, temps[:R], 23, precision=prec, cluster=cluster, atom_threads=P)
+        ctx.advance(12)
+        ctx.advance(np.arange(R) % 5 + 1)
+        x, v = ctx.get_state()
+        state.append((x[:12 * N], v[:12 * N], ctx.energies()[0][:12]))
+        ctx.close()
+    for a, b in zip(*state):
+        np.testing.assert_array_equal(a, b)
