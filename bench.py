@@ -342,7 +342,7 @@ def run_gpu(args, cfg):
         tuned = ctx.config()
     else:
         ctx = make(skin)
-        tuned = ctx.autotune(steps=40)
+        tuned = ctx.autotune(steps=nx if nx > 0 else 40)  # as the cycles run it
     Rtot = ctx.n_rep
     W, K = args.warmup, args.steps
     budgets = make_budgets(cfg, Rtot, W + K, 7 + rank)

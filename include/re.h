@@ -76,7 +76,8 @@ typedef struct re_opts {
   int pair_parity;  /* 0 (default): first pair offset alternates 0,1; 1: random      */
   int nx;           /* steps per replica used by re_advance(c, NULL); default 10      */
   int nbr_capacity; /* neighbours per atom; 0: from the density with a 6-sigma margin */
-  int cell_div;     /* list cells per list radius (1..3); 0: automatic               */
+  int cell_div;     /* cells per list radius (1..3), 0: automatic: the plain path's
+                       list build and the order of sort_interval                */
   int cluster;      /* CTAs cooperating on one replica (1, 2, 3, 4, 8); 0: automatic  */
   int atom_threads; /* threads sharing one atom's neighbour list (1, 2, 4, 8); 0: auto */
   int sort_interval;/* mixed batched path: renumber each replica's atoms in space order
@@ -299,7 +300,7 @@ int re_accept_stats(re_ctx *c, int64_t *attempts, int64_t *accepts);
 /* Shape of the context: replicas, atoms of all replicas, ensembles, pair
  * stats entries (any may be NULL). */
 int re_info(const re_ctx *c, int *n_rep, int64_t *n_atoms, int *n_ens, int *n_pairs);
-/* Launch configuration in use: CTAs per replica, threads per CTA, list cells
+/* Launch configuration in use: CTAs per replica, threads per CTA, cells
  * per list radius, threads per atom (any may be NULL). */
 int re_config(const re_ctx *c, int *cluster, int *threads, int *cell_div, int *atom_threads);
 /* re_config and whether the neighbour lists are kept in shared memory. */
@@ -319,9 +320,10 @@ int re_config_wide(const re_ctx *c, int *wide_n, int *wide_cluster, int *wide_th
                    int *wide_atom_threads);
 /* Times candidate launch configurations (cluster, atom_threads, cell_div,
  * the lists' placement, global or shared memory, and each as one launch or
- * split, see re_opts.wide_launch) over `steps` steps each on a copy of the
- * state and keeps the fastest; the state is restored afterwards.  With
- * per-ensemble launches (re_opts.group_launch) every ensemble's shape is
+ * split, see re_opts.wide_launch) in launches of `steps` steps, as the caller
+ * will make them, on a copy of the state and keeps the fastest; the state is
+ * restored afterwards.  cell_div is varied only while no shape is admitted.
+ * With per-ensemble launches (re_opts.group_launch) every ensemble's shape is
  * tuned on its own launch. */
 int re_autotune(re_ctx *c, int steps);
 /* Queues subsequent work on stream (a cudaStream_t; NULL: legacy default). */

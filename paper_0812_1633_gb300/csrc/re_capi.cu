@@ -37,7 +37,8 @@ using re::set_capacity;
 
 namespace re {
 
-// List cells: nc = floor(L / (rlist / m)) cells per side scanned over a
+// Cells of the plain path's list build (and of the spatial sort):
+// nc = floor(L / (rlist / m)) per side, scanned over a
 // (2m + 1)^3 neighbourhood; cells only pay when 2m + 1 < nc.  m is chosen
 // to minimise candidates per atom plus a per-cell visiting cost.
 void choose_cells(double L, double rlist, int N, int want_m, int* nc_out, int* m_out) {
@@ -1938,8 +1939,10 @@ int re_autotune(re_ctx* c, int steps) {
   ApiRange range_("re_autotune");
   if (!c) return fail(nullptr, RE_EINVAL, "context is NULL");
   if (c->opt.path != RE_PATH_BATCHED) return RE_OK;
-  // each trial starts with a full list build; enough steps that it does not dominate
-  steps = std::max(steps, 40);
+  // launches of as many steps as the caller's, whose fixed parts (start, lists
+  // copied to shared memory, a split launch's ordering) count as they do in use
+  steps = std::max(steps, 1);
+  const int n_warm = (40 + steps - 1) / steps, n_timed = std::max(2, (120 + steps - 1) / steps);
   int rc = status_check(c);
   if (rc) return rc;
   // snapshot everything a trial run changes
@@ -1980,19 +1983,27 @@ int re_autotune(re_ctx* c, int steps) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   c->tuning = true;
-  // One trial: restore the state, build every list of the shape (one step,
-  // untimed), then time `steps` steps with valid lists; best of two.  run(b)
-  // enqueues the launch(es) under test with budgets b.  A trial that
-  // overflowed or failed stopped early: it is never picked.
+  // One trial: restore the state, build every list of the shape (one step) and
+  // run some 40 steps untimed, then time launches of some 120; best of two.
+  // run(b) enqueues the launch(es) under test with budgets b.  The untimed steps
+  // matter: lists built all at once also wear out together, which hides the
+  // wait for the replicas that rebuild more often than others.  (One launch of
+  // 40 steps timed right after the builds picked for 64 x 864 a split launch
+  // with lists in shared memory, 192 us a cycle of 10 steps; one launch with the
+  // lists in global memory takes 180.)  A trial that overflowed or failed
+  // stopped early: it is never picked.
   auto trial = [&](auto run) -> float {
     float ms = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       for (auto& b : bufs)
         cudaMemcpyAsync(b.dev, b.save, b.bytes, cudaMemcpyDeviceToDevice, c->stream);
       cudaMemsetAsync(c->s.valid, 0, 4 * R, c->stream);
-      if (run(d_one) != RE_OK) break;
-      cudaEventRecord(e0, c->stream);
-      if (run(c->d_budget) != RE_OK) break;
+      bool ok = run(d_one) == RE_OK;
+      for (int k = 0; k < n_warm + n_timed && ok; ++k) {
+        if (k == n_warm) cudaEventRecord(e0, c->stream);
+        ok = run(c->d_budget) == RE_OK;
+      }
+      if (!ok) break;
       cudaEventRecord(e1, c->stream);
       if (cudaEventSynchronize(e1) != cudaSuccess) break;
       float t = 0;
@@ -2019,8 +2030,11 @@ int re_autotune(re_ctx* c, int steps) {
       const int e = (int)ei;
       LaunchCfg cbest = c->ecfg[e];
       float cbest_ms = 1e30f;
+      // the cells order the atoms and bound the admission, no more: other
+      // divisions are tried where the automatic one admits no shape
       for (int m = 0; m <= 3; ++m) {
         if (c->opt.cell_div > 0 && m != c->opt.cell_div) continue;
+        if (cbest_ms < 1e30f) break;
         EnsDev& d = c->ens[e];
         int nc = 0, mm = 0;
         choose_cells(d.L, d.rlist, d.N, m, &nc, &mm);
@@ -2057,6 +2071,7 @@ int re_autotune(re_ctx* c, int steps) {
     float best_ms = 1e30f;
   for (int m = 0; m <= 3; ++m) {
     if (c->opt.cell_div > 0 && m != c->opt.cell_div) continue;
+    if (best_ms < 1e30f) break;  // as above
     apply_cells(c, m);
     if (m > 0) {
       bool any = false;

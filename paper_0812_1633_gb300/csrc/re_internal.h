@@ -54,7 +54,8 @@ struct StepConst {
 
 struct EnsHdr {
   int N, R, rep_off, pair_off;  // replicas [rep_off, rep_off + R); stats at pair_off
-  int nc, m;                    // list cells per side (0: all pairs), reach in cells
+  int nc, m;                    // cells per side (0: all pairs) and reach in cells, of the
+                                // plain path's list build and the spatial sort
   int cap;                      // neighbour entries per atom: max over P of P * capsub[P]
   int capsub[4];                // sub-list capacity (multiple of 4) for P = 1, 2, 4, 8
   int shift, parity_mode, xdist;  // xdist: exchange pairs at ladder distance xdist (>= 1)
@@ -154,7 +155,7 @@ struct FreeDev {
 
 struct LaunchCfg {
   int cluster, threads, cell_div, atom_threads;  // CTAs per replica, threads per CTA,
-                                                 // list cells per list radius, threads per atom
+                                                 // cells per list radius, threads per atom
   int lists_smem;  // 1: each CTA's sub-lists in shared memory during a launch (when they fit)
   // Budget mode of a one-ensemble context: the wide_n hottest replicas (by
   // current temperature) run in a second, concurrent launch with clusters of
@@ -166,7 +167,7 @@ struct LaunchCfg {
   int wide_n, wide_cluster, wide_threads, wide_atom_threads;
 };
 
-// Host helpers (re_capi.cu): list cells of an ensemble and neighbour capacities.
+// Host helpers (re_capi.cu): cells of an ensemble and neighbour capacities.
 void choose_cells(double L, double rlist, int N, int want_m, int* nc_out, int* m_out);
 void set_capacity(EnsDev& e, int user_cap);
 // e.kc from L, rc, rlist, skin, dt, tau, shift and N (target T = 1)
