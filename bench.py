@@ -945,13 +945,13 @@ def run_diffusion(args):
 # capture per workload and launch shape (profiles/md_batched_kernel_64x864.md),
 # valid only while the kernel's sources are the ones that were profiled.
 PROFILED_TRAFFIC = {
-    ("c1", (2, 2, 2), "mixed"): {"kernel_sha256_16": "18434b74ee98391d",
-                                 "bytes_per_launch": 14120960 + 768,
+    ("c1", (2, 2, 2), "mixed"): {"kernel_sha256_16": "a4ad8bc1e28300ab",
+                                 "bytes_per_launch": 13372416 + 114432,
                                  # pipe use over the SMs' active cycles (ncu --set full)
-                                 "pipes": {"fma_pct": 26.50, "alu_pct": 43.97, "fp64_pct": 3.81,
-                                           "issue_active_pct": 64.53,
-                                           "smem_wavefronts": 21918819,
-                                           "smem_bank_conflicts": 8731644}},
+                                 "pipes": {"fma_pct": 20.37, "alu_pct": 42.45, "fp64_pct": 4.54,
+                                           "issue_active_pct": 54.64,
+                                           "smem_wavefronts": 18331402,
+                                           "smem_bank_conflicts": 7500934}},
 }
 
 
