@@ -474,8 +474,9 @@ __global__ void exchange_kernel(StateDev S, const EnsDev* __restrict__ ens, int3
 // are the same.  A second barrier makes every CTA's updates visible before the
 // record is written and the attempt counted.  Bound by the counting and the
 // FP64 chain of a pair.  Attempts back to back, with one comparison an element,
-// unrolled, one thread a pair and the factors beside the decision: 17.1 us for
-// 1024 replicas, 141 for 4000, against 24.6 and 209 with a thread a position.
+// unrolled, one thread a pair and the factors beside the decision: 18.5 us for
+// 1024 replicas, 141 for 4000, against 24.6 and 209 with a thread a position
+// (1.4 us of it wait until every CTA of the cluster has started).
 __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ ens,
                                         int32_t* partner_out, uint8_t* acc_out, double* rec,
                                         int rtot) {
@@ -491,6 +492,7 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
   long long* key = reinterpret_cast<long long*>(sh);  // R: T/lam as bit patterns
   int* order = reinterpret_cast<int*>(key + R);       // R: replica at each ladder position
   const int tid = threadIdx.x, nt = blockDim.x;
+  cl.barrier_arrive();  // waited for below: no CTA writes to another before that one has started
   for (int a = tid; a < R; a += nt) {
     const double T = S.T[base + a], lam = S.lam[base + a];
     key[a] = __double_as_longlong(lam == 1.0 ? T : T / lam);
@@ -501,6 +503,7 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
     if (partner_out) partner_out[base + a] = -1;
     if (acc_out) acc_out[base + a] = 0;
   }
+  cl.barrier_wait();
   __syncthreads();
   // G threads (consecutive lanes, G a power of two <= 32) per replica
   int G = 1;
@@ -589,7 +592,8 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
 // and the exponential (several hundred clocks each) only D and exp(D) follow
 // one another, the rest runs beside them.  Bound by that chain and the
 // launch: 5.9 us for 64 replicas (one thread a pair and a bitonic sort: 7.8),
-// 16.6 for 1000 with lam (46.9 on one CTA).  The decision is metropolis(): both
+// 12.4 for 1000 with lam (46.9 on one CTA; 16.6 with every key divided on every
+// CTA).  The decision is metropolis(): both
 // members of a pair evaluate it on the same values in the same order.
 __global__ void __launch_bounds__(512) exchange_raw_kernel(
     int R, const double* __restrict__ T, const double* __restrict__ lam,
@@ -602,10 +606,26 @@ __global__ void __launch_bounds__(512) exchange_raw_kernel(
   long long* key = reinterpret_cast<long long*>(sh);  // R: T/lam as bit patterns
   int* order = reinterpret_cast<int*>(key + R);       // R: replica at each ladder position
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int a = tid; a < R; a += nt) key[a] = __double_as_longlong(lam ? T[a] / lam[a] : T[a]);
-  __syncthreads();
   const int per = (R + C - 1) / C;
   const int a0 = min(R, cr * per), a1 = min(R, a0 + per);
+  // no CTA writes to another before that one has started
+  if (C > 1) cl.barrier_arrive();
+  if (lam && C > 1) {
+    // every CTA divides for its own slice and hands the keys to the others: all
+    // of them on every CTA would occupy its FP64 unit for several microseconds
+    const int a = a0 + tid;
+    long long k = a < a1 ? __double_as_longlong(T[a] / lam[a]) : 0;
+    cl.barrier_wait();
+    for (int b = a; b < a1; b += nt) {
+      if (b != a) k = __double_as_longlong(T[b] / lam[b]);
+      for (int rk = 0; rk < C; ++rk) *cl.map_shared_rank(key + b, rk) = k;
+    }
+    cl.sync();
+  } else {
+    for (int a = tid; a < R; a += nt) key[a] = __double_as_longlong(lam ? T[a] / lam[a] : T[a]);
+    if (C > 1) cl.barrier_wait();
+    __syncthreads();
+  }
   // G threads (consecutive lanes, G a power of two <= 32) per replica
   int G = 1;
   while (G < 32 && G * 2 * per <= nt) G *= 2;
