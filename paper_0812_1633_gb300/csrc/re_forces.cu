@@ -169,7 +169,10 @@ cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixe
   const size_t smem = (size_t)N * 16;
   auto fn = mixed ? direct_force_kernel<true> : direct_force_kernel<false>;
   if (smem > 40 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the largest any call may ask for (beside the kernel's own 2.2 KB): a limit
+    // of this call's size could undercut another thread's launch
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               std::max((int)smem, 232448 - 4096));
     if (e != cudaSuccess) return e;
   }
   const double i2 = 1.0 / (K.lam64 * K.lam64);  // (2^64 / L)^2

@@ -1119,12 +1119,7 @@ cudaError_t launch_exchange(const StateDev& s, const EnsDev* d_ens, int n_ens, i
     // one cluster per ensemble: about 128 replicas per CTA, at most 8 CTAs
     const int C = std::min(8, (max_r + 127) / 128);
     const int threads = 512;
-    const size_t smem = (size_t)max_r * (sizeof(long long) + sizeof(int));
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(exchange_cluster_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const size_t smem = (size_t)max_r * (sizeof(long long) + sizeof(int));  // at most 4096: 48 KB
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3((unsigned)(n_ens * C));
     lc.blockDim = dim3((unsigned)threads);
@@ -1140,12 +1135,7 @@ cudaError_t launch_exchange(const StateDev& s, const EnsDev* d_ens, int n_ens, i
     return cudaLaunchKernelEx(&lc, exchange_cluster_kernel, s, d_ens, d_partner, d_acc, d_rec,
                               rtot);
   }
-  const size_t smem = exchange_smem_bytes(max_r);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(exchange_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const size_t smem = exchange_smem_bytes(max_r);  // 13 KB at most
   // eight lanes rank a replica of up to 64, two one of 256
   const int threads = std::min(512, ((max_r * 8 + 31) / 32) * 32);
   exchange_kernel<<<n_ens, threads, smem, st>>>(s, d_ens, d_partner, d_acc, d_rec, rtot);
@@ -1207,12 +1197,7 @@ cudaError_t launch_exchange_raw(int R, const double* T, const double* lam, const
                                 cudaStream_t st) {
   // about 128 replicas per CTA, at most 8 CTAs; one CTA needs no cluster launch
   const int C = std::min(8, (R + 127) / 128);
-  const size_t smem = (size_t)R * (sizeof(long long) + sizeof(int));
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(exchange_raw_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const size_t smem = (size_t)R * (sizeof(long long) + sizeof(int));  // R at most 4096: 48 KB
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)C);
   lc.blockDim = dim3(512);
