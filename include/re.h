@@ -341,7 +341,8 @@ void re_destroy(re_ctx *c);
 /* One exchange attempt over R <= 4096 replicas (Implementation section), as
  * in re_exchange: T, U device arrays (R doubles); outputs T_out (R doubles,
  * new temperatures), partner (R int32, -1 if unpaired), accepted (R uint8),
- * vscale (R doubles, sqrt(T_new/T_old) or 1).  T must hold distinct positive values. */
+ * vscale (R doubles, sqrt(T_new/T_old) or 1).  T must hold distinct positive values.
+ * In place: an output array may be an input array (T_out = T). */
 int re_exchange_device(int R, const double *T, const double *U, uint64_t seed, int64_t attempt,
                        int parity_mode, double *T_out, int32_t *partner, uint8_t *accepted,
                        double *vscale, void *stream);
@@ -351,7 +352,7 @@ int re_exchange_device(int R, const double *T, const double *U, uint64_t seed, i
  * re_exchange_device, plus lam_out (NULL allowed) = the swapped scales and
  * uscale (NULL allowed) = lam_new/lam_old per replica.  Keys T/lam must be
  * distinct and positive.  The same decisions as re_exchange for the same
- * state. */
+ * state.  In place as re_exchange_device (T_out = T, lam_out = lam). */
 int re_exchange_device_h(int R, const double *T, const double *lam, const double *U,
                          uint64_t seed, int64_t attempt, int parity_mode, int distance,
                          double *T_out, double *lam_out, int32_t *partner, uint8_t *accepted,

@@ -596,10 +596,9 @@ __global__ void exchange_cluster_kernel(StateDev S, const EnsDev* __restrict__ e
 // CTA).  The decision is metropolis(): both
 // members of a pair evaluate it on the same values in the same order.
 __global__ void __launch_bounds__(512) exchange_raw_kernel(
-    int R, const double* __restrict__ T, const double* __restrict__ lam,
-    const double* __restrict__ U, uint64_t seed, int64_t attempt, int mode, int distance,
-    double* T_out, double* lam_out, int32_t* partner, uint8_t* acc, double* vscale,
-    double* uscale) {
+    int R, const double* T, const double* lam, const double* U, uint64_t seed, int64_t attempt,
+    int mode, int distance, double* T_out, double* lam_out, int32_t* partner, uint8_t* acc,
+    double* vscale, double* uscale) {
   extern __shared__ __align__(16) unsigned char sh[];
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), cr = (int)cl.block_rank();
@@ -644,12 +643,18 @@ __global__ void __launch_bounds__(512) exchange_raw_kernel(
     __syncthreads();
   const int p = pair_offset(mode, seed, attempt);
   const int d = max(1, distance);
-  for (int q = a0 + tid; q < a1; q += nt) {
-    const int m = order[q], qb = ladder_partner(q, R, p, d);
+  // a slice has at most 4096 / 8 replicas: one each for the 512 threads
+  const int q = a0 + tid;
+  const bool mine = q < a1;
+  int m = 0, other = -1;
+  double Tn = 0.0, ln = 1.0, vs = 1.0, us = 1.0;
+  bool ok = false;
+  if (mine) {
+    m = order[q];
+    const int qb = ladder_partner(q, R, p, d);
     const double Tm = T[m], lm = lam ? lam[m] : 1.0;
-    double Tn = Tm, ln = lm, vs = 1.0, us = 1.0;
-    int other = -1;
-    bool ok = false;
+    Tn = Tm;
+    ln = lm;
     if (qb >= 0) {
       other = order[qb];
       const double To = T[other], lo = lam ? lam[other] : 1.0;
@@ -665,6 +670,15 @@ __global__ void __launch_bounds__(512) exchange_raw_kernel(
         us = ratio;
       }
     }
+  }
+  // outputs may lie over inputs (T_out over T, lam_out over lam, ...): every
+  // replica's inputs, which two threads read, are read before any result is
+  // written
+  if (C > 1)
+    cl.sync();
+  else
+    __syncthreads();
+  if (mine) {
     T_out[m] = Tn;
     if (lam_out) lam_out[m] = ln;
     partner[m] = other;
@@ -672,7 +686,6 @@ __global__ void __launch_bounds__(512) exchange_raw_kernel(
     vscale[m] = vs;
     if (uscale) uscale[m] = us;
   }
-  if (C > 1) cl.sync();  // no CTA leaves while another may still write its order
 }
 
 // Exchange results decided elsewhere (a ladder sharded over several
