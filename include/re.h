@@ -81,7 +81,8 @@ typedef struct re_opts {
   int cluster;      /* CTAs cooperating on one replica (1, 2, 3, 4, 8); 0: automatic  */
   int atom_threads; /* threads sharing one atom's neighbour list (1, 2, 4, 8); 0: auto */
   int sort_interval;/* mixed batched path: renumber each replica's atoms in space order
-                       every this many steps (0: every 200; < 0: never).  Results
+                       every this many steps (0: every 200; < 0: never), and after a
+                       re_set_state whose numbering does not follow space.  Results
                        differ only in summation order; atom order in the API is
                        always the original one. */
   int exch_distance;/* exchange pairs at ladder distance d (default 1: nearest

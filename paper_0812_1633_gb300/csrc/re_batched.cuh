@@ -284,6 +284,19 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       // the FP64 pair loop's notes overlie the screening vectors
       if (FP64 && P >= 4) __syncthreads();
     }
+    if (P > 1) {
+      // a sub-list that overflowed: its atom's entries dealt out evenly
+      const uint32_t over = __ballot_sync(0xffffffffu, cnt > cap_sub);
+      if (over) {
+        const bool redo = own && ((over >> (lane & ~(P - 1))) & ((1u << P) - 1u)) != 0u;
+        const int n = deal_sublist<P>(i, q, redo, hi_of, N, K.rl2u, nb, mycol, ncols, cap_sub, &overflow);
+        if (redo) cnt = n;
+      }
+    }
+    if (cnt > cap_sub) {
+      overflow |= kStOverflow;
+      cnt = cap_sub;  // whole blocks
+    }
     if (own) {
 #pragma unroll
       for (int j = 0; j < ND; ++j)

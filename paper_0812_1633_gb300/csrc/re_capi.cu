@@ -1659,6 +1659,39 @@ int re_get_state(re_ctx* c, double* x, double* v) {
   return RE_OK;
 }
 
+namespace {
+
+// Whether atoms that follow one another in x mostly lie within the list radius
+// of one another (a sample of about a thousand pairs over all replicas).  Where
+// they don't -- any order that does not follow space -- the atoms are renumbered
+// before the next lists instead of at the next interval: 64 x 4000 atoms in
+// random order 64 us a step instead of 79, 8 x 2048 atoms of four slabs in turn
+// (whose sub-lists overflow and are dealt) 15 instead of 39.  An order that
+// follows space is kept: the sort costs 20 to 50 us, and its cells of about 30
+// atoms are a coarser order than a lattice's rows.
+bool numbered_in_space(const re_ctx* c, const double* x) {
+  const int per = std::max(1, 1024 / c->n_rep);
+  int near = 0, n = 0;
+  for (int r = 0; r < c->n_rep; ++r) {
+    const EnsDev& e = c->ens[c->reps[r].ens];
+    const double* xr = x + 3 * (size_t)c->reps[r].atom_off;
+    for (int k = 0; k < per; ++k) {
+      const int i = (int)(((int64_t)k * (e.N - 1) / per + 7 * r) % (e.N - 1));
+      double r2 = 0.0;
+      for (int d = 0; d < 3; ++d) {
+        double s = (xr[3 * (i + 1) + d] - xr[3 * i + d]) * e.kc.inv_l;
+        s -= std::nearbyint(s);
+        r2 += s * s * e.L * e.L;
+      }
+      near += r2 < e.rlist * e.rlist ? 1 : 0;
+      ++n;
+    }
+  }
+  return 2 * near >= n;
+}
+
+}  // namespace
+
 int re_set_state(re_ctx* c, const double* x, const double* v) {
   if (!c) return fail(nullptr, RE_EINVAL, "context is NULL");
   const size_t n3 = 3 * (size_t)c->n_atoms;
@@ -1669,6 +1702,7 @@ int re_set_state(re_ctx* c, const double* x, const double* v) {
     e = re::launch_import_state(c->s, c->d_ens, c->d_rep, c->n_rep, c->d_io, nullptr, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "import");
     RE_CUDA(c, cudaStreamSynchronize(c->stream), "synchronise");
+    if (c->sort_every > 0 && !numbered_in_space(c, x)) c->since_sort = c->sort_every;
   }
   if (v) {
     RE_CUDA(c, cudaMemcpyAsync(c->d_io, v, 8 * n3, cudaMemcpyHostToDevice, c->stream), "write v");

@@ -502,17 +502,14 @@ __device__ __forceinline__ void cta_screen_vectors(PosFn pos_hi, int N, uint4* h
   __syncthreads();
 }
 
-// The end of a sub-list: overflow and coincident atoms (closer than L / 2^32:
-// the pair loop cannot give their force a direction) reported, the last block
-// filled up with the atom's own index.
+// The end of a sub-list: coincident atoms (closer than L / 2^32: the pair loop
+// cannot give their force a direction) reported, the last block filled up with
+// the atom's own index.  cnt, which the caller compares with cap_sub, is
+// returned as it is.
 __device__ __forceinline__ int finish_sublist(int cnt, uint2 blk, uint2* out, int i,
-                                              bool coincident, int cap_sub, int* overflow) {
-  if (coincident) *overflow |= kStNumeric;
-  if (cnt > cap_sub) {
-    *overflow |= kStOverflow;
-    return cap_sub;  // whole blocks
-  }
-  if (cnt & 3) {
+                                              bool coincident, int cap_sub, int* status) {
+  if (coincident) *status |= kStNumeric;
+  if (cnt <= cap_sub && (cnt & 3)) {
     for (int k = cnt; k & 3; ++k) {
       blk.x = __funnelshift_r(blk.x, blk.y, 16);
       blk.y = __byte_perm(blk.y, (uint32_t)i, 0x5432);
@@ -520,6 +517,43 @@ __device__ __forceinline__ int finish_sublist(int cnt, uint2 blk, uint2* out, in
     *out = blk;
   }
   return cnt;
+}
+
+// The sub-lists of atoms whose neighbours the builds below spread too unevenly
+// over the lanes: they go by the atoms' numbers, so an order that puts the
+// neighbours of an atom into one residue class (the atoms of P spatial domains
+// taken in turn) gives one lane all of them.  Here the entries found so far
+// decide: the k-th goes to lane k % P, the P counts differ by one at most, and
+// an atom overflows only when its whole list does.  `redo` (equal on an atom's
+// lanes) says whose lists are made; the order depends on the atom and P alone.
+// Whole warps; some 35 instructions per P atoms, run when a sub-list overflowed.
+template <int P, class PosFn>
+__device__ __forceinline__ int deal_sublist(int i, int q, bool redo, PosFn pos_hi, int N, float rl2u,
+                                            uint16_t* nb, uint32_t col, uint32_t ncols, int cap_sub,
+                                            int* status) {
+  const int group = threadIdx.x & 31 & ~(P - 1);  // the atom's first lane
+  const Hi3 pi = redo ? pos_hi(i) : Hi3{0u, 0u, 0u};
+  int cnt = 0, total = 0;
+  uint2 blk = make_uint2(0u, 0u);  // the last four entries
+  uint2* out = reinterpret_cast<uint2*>(nb) + col;
+#pragma unroll 1
+  for (int j0 = 0; j0 < N; j0 += P) {
+    const int j = j0 + q;
+    const bool hit = redo && j < N && j != i && sep2_hi(pi, pos_hi(j)) < rl2u;
+    uint32_t b = (__ballot_sync(0xffffffffu, hit) >> group) & ((1u << P) - 1u);
+    const int k = (q - total) & (P - 1);  // which of these hits is this lane's
+    total += __popc(b);
+    for (int s = 0; s < k; ++s) b &= b - 1;
+    if (b == 0u) continue;
+    blk.x = __funnelshift_r(blk.x, blk.y, 16);
+    blk.y = __byte_perm(blk.y, (uint32_t)(j0 + __ffs(b) - 1), 0x5432);
+    if ((cnt & 3) == 3) {
+      if (cnt < cap_sub) *out = blk;
+      out += ncols;
+    }
+    ++cnt;
+  }
+  return finish_sublist(cnt, blk, out, i, false, cap_sub, status);
 }
 
 // The list of a small replica, by testing every atom: lane q takes the atoms j
@@ -532,7 +566,7 @@ constexpr int kDirectBuild = 256;
 template <int P, class PosFn>
 __device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosFn pos_hi, int N,
                                                     float rl2u, uint16_t* nb, uint32_t col,
-                                                    uint32_t ncols, int cap_sub, int* overflow) {
+                                                    uint32_t ncols, int cap_sub, int* status) {
   if (!own) return 0;
   const Hi3 pi = pos_hi(i);
   int cnt = 0;
@@ -553,7 +587,7 @@ __device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosF
     if (full) out += ncols;
     cnt += add ? 1 : 0;
   }
-  return finish_sublist(cnt, blk, out, i, coincident, cap_sub, overflow);
+  return finish_sublist(cnt, blk, out, i, coincident, cap_sub, status);
 }
 
 // Sub-list of lane q (of P) of atom i, by whole warps (every lane of the warp
@@ -577,7 +611,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
                                              const uint4* hk, const uint2* box, uint8_t* act,
                                              float rl2u, uint16_t* nb, uint32_t col,
                                              uint32_t ncols, uint16_t* raw, uint32_t rcol,
-                                             uint32_t rncols, int cap_sub, int* overflow) {
+                                             uint32_t rncols, int cap_sub, int* status) {
   const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
   if (!__any_sync(0xffffffffu, own)) return 0;
   const Hi3 pi = own ? pos_hi(i) : Hi3{0u, 0u, 0u};
@@ -746,7 +780,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
   // of the atom's lanes, the one whose columns hold the atom met it once
   const bool self = P == 1 || (P == 2 && (t & 1) == (i & 1)) || (P == 4 && t == (i & 3)) ||
                     (P == 8 && t == (i & 3) && (g & 1) == ((i >> 3) & 1));
-  return finish_sublist(cnt, blk, out, i, zeros > (self ? 1 : 0), cap_sub, overflow);
+  return finish_sublist(cnt, blk, out, i, zeros > (self ? 1 : 0), cap_sub, status);
 }
 
 // Mixed-precision forces of atom i from this lane's sub-list; see mixed_pair2.
