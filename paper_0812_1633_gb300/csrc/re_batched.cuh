@@ -279,8 +279,9 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       cta_screen_vectors(hi_of, N, sm.hk, sm.box);
       cnt = build_sublist<P>(i, own, i0 + warp * (32 / P), hi_of, N, sm.hk, sm.box,
                              sm.act + warp * row_list_bytes(N), K.rl2u, nb, mycol, ncols,
-                             S.raw + rd.nbr_off, (uint32_t)(i * P + q), (uint32_t)(N * P), cap_sub,
-                             &overflow);
+                             S.raw ? S.raw + rd.nbr_off : nbg + (size_t)N * P * cap_sub,
+                             (uint32_t)(i * P + q), (uint32_t)(N * P),
+                             S.raw ? cap_sub / 4 : list_notes(E.cap, cap_sub, P), cap_sub, &overflow);
       // the FP64 pair loop's notes overlie the screening vectors
       if (FP64 && P >= 4) __syncthreads();
     }

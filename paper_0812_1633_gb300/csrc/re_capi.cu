@@ -384,6 +384,17 @@ int upload_tables(re_ctx* c) {
 }
 
 // Allocate device memory for the current ens/reps tables.
+// Whether a screened list build (see re_batched.cuh) of some launch shape would
+// find next to no room for its notes in the list array: sparse systems and
+// capacities given by the caller.  An array of their own then holds them.
+bool notes_need_room(const re_ctx* c) {
+  if (c->opt.path != RE_PATH_BATCHED) return false;
+  for (const EnsDev& e : c->ens)
+    for (int k = 0; k < 3; ++k)
+      if (e.N > (re::kDirectBuild << k) && re::list_notes(e.cap, e.capsub[k], 1 << k) < 4) return true;
+  return false;
+}
+
 int allocate(re_ctx* c) {
   const size_t A = (size_t)c->n_atoms, R = (size_t)c->n_rep, E = c->ens.size();
   StateDev& s = c->s;
@@ -393,7 +404,7 @@ int allocate(re_ctx* c) {
       (rc = dalloc(c, &s.fx, A)) || (rc = dalloc(c, &s.fy, A)) || (rc = dalloc(c, &s.fz, A)) ||
       (rc = dalloc(c, &s.rx, A)) || (rc = dalloc(c, &s.ry, A)) || (rc = dalloc(c, &s.rz, A)) ||
       (rc = dalloc(c, &s.ncnt, 8 * A)) || (rc = dalloc(c, &s.nbr, (size_t)c->n_nbr)) ||
-      (c->opt.path == RE_PATH_BATCHED && (rc = dalloc(c, &s.raw, (size_t)c->n_nbr))) ||
+      (notes_need_room(c) && (rc = dalloc(c, &s.raw, (size_t)c->n_nbr))) ||
       (rc = dalloc(c, &s.T, R)) || (rc = dalloc(c, &s.U, 4 * R)) || (rc = dalloc(c, &s.vscale, R)) ||
       (rc = dalloc(c, &s.lam, R)) || (rc = dalloc(c, &s.fscale, R)) ||
       (rc = dalloc(c, &s.step, R)) || (rc = dalloc(c, &s.nreb, R)) ||

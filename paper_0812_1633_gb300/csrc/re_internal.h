@@ -93,13 +93,24 @@ struct RepDev {
   int64_t nbr_off;
 };
 
+// Replicas of at most this many atoms per thread of an atom have their lists built
+// by testing every atom, larger ones by screening (re_md.cuh).
+constexpr int kDirectBuild = 256;
+
+// Notes (candidate masks, 8 bytes each) that the screened list build of a lane
+// can keep in the part of its replica's list array that a layout of P threads per
+// atom leaves unused (the array holds the largest layout, P = 8).
+__host__ __device__ inline int list_notes(int cap, int cap_sub, int P) {
+  return (cap - P * cap_sub) / (4 * P);
+}
+
 struct StateDev {
   uint64_t *qx, *qy, *qz;
   double *vx, *vy, *vz, *fx, *fy, *fz;
   uint32_t *rx, *ry, *rz;
   int32_t* ncnt;
   uint16_t* nbr;
-  uint16_t* raw;  // as nbr: candidates that passed a list build's screening (scratch)
+  uint16_t* raw;  // as nbr: notes of the list builds, where list_notes() finds no room (else null)
   double *T, *U, *K, *econs, *vscale;
   double *lam, *fscale;  // per replica: potential scale; pending force factor (null: 1)
   int64_t *step, *nreb;

@@ -559,10 +559,8 @@ __device__ __forceinline__ int deal_sublist(int i, int q, bool redo, PosFn pos_h
 // The list of a small replica, by testing every atom: lane q takes the atoms j
 // with j % P == q, in increasing order.  Below kDirectBuild atoms a lane this
 // costs less than the screening and its notes (20 instructions an atom, no
-// divergence): with P = 4 at 500 atoms 19.6 thousand clocks a build against
+// divergence; re_internal.h): with P = 4 at 500 atoms 19.6 thousand clocks a build against
 // 23.5; with P = 2 at 864 atoms, past the line, 58 against 53.
-constexpr int kDirectBuild = 256;
-
 template <int P, class PosFn>
 __device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosFn pos_hi, int N,
                                                     float rl2u, uint16_t* nb, uint32_t col,
@@ -594,8 +592,8 @@ __device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosF
 // calls; `own` says whether it holds an atom; iw: the warp's first atom): entry
 // k at element ((k / 4) * ncols + col) * 4 + k % 4 of nb, written four at a
 // time, the last four filled up with the atom's own index.  raw, rcol, rncols:
-// room for the notes, one 8-byte word each, laid out likewise.  act: this warp's
-// row list.
+// room for max_notes >= 1 notes, one 8-byte word each, laid out likewise.  act: this
+// warp's row list.
 //
 // Tile v of a row (v = 0..3) holds the atoms t + 8 v + 4 c at columns 2 t + c,
 // and lane 4 g + t gets columns 2 t, 2 t + 1 of the tile rows g and g + 8: it
@@ -611,7 +609,8 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
                                              const uint4* hk, const uint2* box, uint8_t* act,
                                              float rl2u, uint16_t* nb, uint32_t col,
                                              uint32_t ncols, uint16_t* raw, uint32_t rcol,
-                                             uint32_t rncols, int cap_sub, int* status) {
+                                             uint32_t rncols, int max_notes, int cap_sub,
+                                             int* status) {
   const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
   if (!__any_sync(0xffffffffu, own)) return 0;
   const Hi3 pi = own ? pos_hi(i) : Hi3{0u, 0u, 0u};
@@ -769,7 +768,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
       const uint32_t w = mk[0];
 #pragma unroll
       for (int y = 0; y + 1 < NM; ++y) mk[y] = mk[y + 1];
-      if (__any_sync(0xffffffffu, nm == cap_sub / 4)) drain();
+      if (__any_sync(0xffffffffu, nm == max_notes)) drain();
       // the row of each byte from the top, lowest byte first
       const uint32_t sel = P == 1 ? x * 0x1111u : (P == 2 ? 0x1100u + x * 0x2222u : 0x3210u);
       if (w) rawp[(size_t)nm++ * rncols] = make_uint2(w, __byte_perm(rows4, 0, sel));
