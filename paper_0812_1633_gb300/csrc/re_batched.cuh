@@ -682,7 +682,7 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
           if (FP64) {
             v[j] *= sc;
           } else {
-            vq[j] = __double2ll_rn((double)vq[j] * sc);
+            vq[j] = vfix_scale(vq[j], sc);  // as a pending factor
           }
         }
       }
