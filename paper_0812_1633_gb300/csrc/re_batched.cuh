@@ -356,8 +356,10 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       const float ax = group_sum<P>(lo2(a.fx) + hi2(a.fx)), ay = group_sum<P>(lo2(a.fy) + hi2(a.fy)),
                   az = group_sum<P>(lo2(a.fz) + hi2(a.fz));
       float ae = 0.0f;
-      if (energy)  // uniform flag
-        ae = group_sum<P>(lo2(a.e) + hi2(a.e)) - ucf * group_sum<P>(lo2(a.n) + hi2(a.n));
+      if (energy) {  // uniform flag
+        ae = group_sum<P>(lo2(a.e) + hi2(a.e));
+        ae = fmaf(ae, K.eu, ae * K.eul) - ucf * group_sum<P>(lo2(a.n) + hi2(a.n));
+      }
       if (own) {
         if (!isfinite(ax) || !isfinite(ay) || !isfinite(az)) st |= kStNumeric;
         if (energy && q == 0) {

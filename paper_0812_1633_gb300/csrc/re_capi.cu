@@ -240,14 +240,7 @@ void finish_ens(EnsDev& e) {
   k.rl2u = (float)(rlu * rlu);
   const double hu = 0.5 * e.skin * (1.0 - 1e-6) / k.lam32;
   k.half2u = (float)(hu * hu);
-  {
-    // (2^32 / L)^2 = kappa 2^e: 2^e scales 1/r^2 in the pair loop, kappa in [0.5, 1)
-    int ex = 0;
-    const double kappa = std::frexp(1.0 / (k.lam32 * k.lam32), &ex);
-    k.cs = (float)-std::ldexp(1.0, ex);
-    k.c3 = (float)(2.0 * kappa * kappa * kappa);
-    k.f24 = 24.0 * kappa * kappa * kappa * kappa;
-  }
+  set_pair_constants(k);
   k.nf = 3 * e.N - 3;
   k.c_th = e.tau > 0.0 ? std::exp(-e.dt / e.tau) : 1.0;
   const double omc = e.tau > 0.0 ? -std::expm1(-e.dt / e.tau) : 0.0;  // 1 - c, no cancellation

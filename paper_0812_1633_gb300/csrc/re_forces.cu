@@ -32,8 +32,8 @@ __global__ void __launch_bounds__(256) direct_fix_kernel(const double* __restric
 // and, in the last CTA to finish, over the CTAs.
 template <bool MIXED>
 __global__ void __launch_bounds__(512) direct_force_kernel(DirectScratch s, int N, StepConst K,
-                                                           Fp64Const c, double unit, int cap,
-                                                           double* __restrict__ f,
+                                                           Fp64Const c, double unit, double eunit,
+                                                           int cap, double* __restrict__ f,
                                                            double* __restrict__ U) {
   extern __shared__ __align__(16) uint4 hi[];
   __shared__ double esum[16];
@@ -70,12 +70,13 @@ __global__ void __launch_bounds__(512) direct_force_kernel(DirectScratch s, int 
                        ez = (double)(long long)(q.z - pi.z);
           if (!(fma(ex, ex, fma(ey, ey, ez * ez)) < c.rc2)) return;
         }
-        const float v = rcp_approx(r2) * K.cs, v2 = v * v, q = v2 * v * K.c3, v4 = v2 * v2;
-        const float fs = fmaf(q, v4, v4);
+        // rounded to nearest: the approximate one is off by 4e-9 in the mean, s^7 by 3e-8
+        const float v = __frcp_rn(r2) * K.cs, v2 = v * v, v3 = v2 * v, v4 = v2 * v2;
+        const float u = fmaf(v3, K.c3, K.c1), fs = v4 * u;
         gx = fmaf(fs, dx, gx);
         gy = fmaf(fs, dy, gy);
         gz = fmaf(fs, dz, gz);
-        ge = fmaf(q, q + 2.0f, ge);
+        ge = fmaf(v3 * K.c3, u + K.c1, ge);
         gn += 1.0f;
       } else {
         fp64_pair<true>(pi, full(j), ph, edge, c, a);
@@ -110,7 +111,7 @@ __global__ void __launch_bounds__(512) direct_force_kernel(DirectScratch s, int 
     // the four sums, halving what a lane holds with the distance: lanes 0-7 end
     // with F_x, 8-15 with F_y, 16-23 with F_z, 24-31 with the energy
     double v[4] = {MIXED ? (double)gx : a.fx, MIXED ? (double)gy : a.fy, MIXED ? (double)gz : a.fz,
-                   MIXED ? (double)ge - K.uc * (double)gn : a.e};
+                   MIXED ? (double)ge * eunit - K.uc * (double)gn : a.e};
     const bool h16 = lane & 16, h8 = lane & 8;
     double p = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
     double q = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
@@ -179,7 +180,8 @@ cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixe
   const Fp64Const c{-2.0 * i2 * i2 * i2, K.rc2 * i2, K.uc};
   // of the pair sums: see lj2 and fp64_pair
   const double unit = mixed ? K.f24 * K.lam32 : 24.0 * i2 * i2 * i2 * (i2 * K.lam64);
-  fn<<<(N + W - 1) / W, 32 * W, smem, st>>>(s, N, K, c, unit, cap, f, U);
+  const double eunit = 1.0 / ((double)K.c1 * K.c1);
+  fn<<<(N + W - 1) / W, 32 * W, smem, st>>>(s, N, K, c, unit, eunit, cap, f, U);
   return cudaGetLastError();
 }
 

@@ -15,6 +15,7 @@
 //             nreb, status, valid
 //   per ensemble: attempt counter; per sorted pair position: attempts, accepts
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -40,11 +41,13 @@ struct StepConst {
   double lam32, lam64, inv_l, dtq, hdt, inv_hdt, uc, rc2, c_th, kbar;
   double kbar1, af1, bf1, gf1;  // kbar = kbar1 T, af = af1 T, bf = bf1 sqrt(T), gf = gf1 / sqrt(T)
   double lamv;                  // the replica's potential scale (set_potential_scale)
-  double f24;                   // 24 kappa^4
+  double f24;                   // 24 kappa^4 / c1
   double rc2x;                  // rc^2 in units (L / 2^42)^2 (exact cutoff test, mixed path)
   float hlf;                    // FP32 half-kick factor per unit of the mixed pair sums, times lamv
   float rc2u, rl2u, half2u;
-  float cs, c3;                 // mixed pair forces: cs = -2^k, c3 = 2 kappa^3, (2^32 / L)^2 = kappa 2^k
+  // mixed pair sums (set_pair_constants), (2^32 / L)^2 = kappa 2^k: cs = -2^k,
+  // c3 / c1 = 2 kappa^3, eu + eul = 1 / c1^2
+  float cs, c1, c3, eu, eul;
   float rc2u_lo, rc2u_hi;       // rc2u (1 -+ 2e-6): the band decided on 42-bit separations
   // thermostat constants of the mixed path (used in FP32): c - 1,
   // (1 - c) Kbar / Nf, 2 sqrt(c (1 - c) Kbar / Nf), sqrt(c Nf / ((1 - c) Kbar))
@@ -70,11 +73,40 @@ struct EnsDev : EnsHdr {
   StepConst kc;  // filled by finish_ens (host) once the fields above are set
 };
 
+// The constants of the mixed pair sums, from lam32 (host).  The force of a pair is
+// 24 (2^k kappa)^4 s^4 (1 + 2 kappa^3 s^3) / c1 times c1: only the ratio c3 / c1
+// counts, f24 and eu take c1 out again.  c1 is any float in [0.5, 1): the first of
+// a scattered sequence whose product with 2 kappa^3 lies within 1e-9 of a float, or
+// the best of 256.  A rounded 2 kappa^3 itself (c1 = 1) is up to 6e-8 off and tilts
+// the r^-14 against the r^-8 part of every pair: 3.4e-8 in boxes of 256 and 2048
+// atoms, 5e-8 in the energies of hot replicas there; now 1e-8 (and 2e-8 at most in
+// other boxes: the approximate reciprocal).  (One rounded (2^32 / L)^2 to the third
+// and seventh power: 1e-8 in those two, 1.3e-7 in boxes of 500 atoms.)
+inline void set_pair_constants(StepConst& k) {
+  int ex = 0;
+  const double kappa = std::frexp(1.0 / (k.lam32 * k.lam32), &ex);  // [0.5, 1)
+  const double k3 = 2.0 * kappa * kappa * kappa;
+  double best = 1.0;
+  for (uint32_t i = 0; i < 256 && best > 1e-9; ++i) {
+    const double c1 = 0.5 + ((i * i * 0x9E3779u + i * 0x3C6EF3u) & 0x7FFFFFu) * 0x1.0p-24;
+    const double c3 = k3 * c1, off = std::fabs((double)(float)c3 / c3 - 1.0);
+    if (off >= best) continue;
+    best = off;
+    k.c1 = (float)c1;
+    k.c3 = (float)c3;
+  }
+  const double e = 1.0 / ((double)k.c1 * k.c1);
+  k.eu = (float)e;
+  k.eul = (float)(e - (double)k.eu);
+  k.cs = (float)-std::ldexp(1.0, ex);
+  k.f24 = 24.0 * kappa * kappa * kappa * kappa / (double)k.c1;
+}
+
 // The constants of StepConst that depend on the replica's potential scale
 // (its Hamiltonian is K + lam U_LJ: forces and U scale by lam).
 __host__ __device__ inline void set_potential_scale(StepConst& k, double lam) {
   k.lamv = lam;
-  // the mixed pair sums are in units of 24 (2^k)^4 s^4 d, s = 1/r^2 in sigma units
+  // the mixed pair sums are in units of c1 (2^k)^4 s^4 d, s = 1/r^2 in sigma units
   k.hlf = (float)(k.hdt * k.lam32 * lam * k.f24);
 }
 

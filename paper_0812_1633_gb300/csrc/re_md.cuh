@@ -123,8 +123,7 @@ __device__ __forceinline__ float sep2_hi(Hi3 a, Hi3 b) {
 // Two list entries are taken at a time, as packed f32x2 instructions (21
 // instead of 28 issued instructions per entry), without a branch per pair:
 // with q = -2 s^3 the force is fs = 24 s^4 (1 + q) (the factor 24 is part of
-// StepConst::hlf), multiplied by 1 inside the cutoff and 0 outside, and the
-// pair energy is q (q + 2).
+// StepConst::hlf) and the pair energy q (q + 2); outside the cutoff s is 0.
 //
 // The cutoff test.  The force is truncated at rc (Example section), so it
 // jumps there by F(rc) ~ 0.04: a pair put on the wrong side of rc costs its
@@ -181,7 +180,7 @@ __device__ __forceinline__ float min3_abs(float a, float b, float c) {
 
 struct PairAcc {
   f32x2 fx, fy, fz;  // force sums over the even and the odd entries
-  f32x2 e, n;        // ENERGY: pair energies, pairs counted inside
+  f32x2 e, n;        // ENERGY: pair energies (times c1^2), pairs counted inside
   float tmin;        // smallest |r^2 - rc^2 (1 + 2e-6)| met
 };
 
@@ -198,15 +197,18 @@ __device__ __forceinline__ bool inside_cutoff_42(uint4 pi, uint4 pj, double x42)
   return fma(dx, dx, fma(dy, dy, dz * dz)) < x42;
 }
 
-// q and s^4 (1 + q) of two pairs from their r^2, s = -(2^k / r^2), q = c3 s^3.
-// The scale 2^k (cs, exact) keeps the powers in range; the one rounded constant
-// c3 enters once (a rounded scale would enter seven times).
-__device__ __forceinline__ void lj2(f32x2 r2, f32x2 cs, f32x2 c3, f32x2& q, f32x2& fs) {
+// Of two pairs from their r^2, with s = cs / r^2 and u = c1 + c3 s^3 = c1 (1 + q):
+// the force s^4 u, c1 q and c1 (q + 2).  The scale 2^k in cs (exact) keeps the
+// powers in range; c3 / c1, the one constant of the force that cannot be exact, is
+// off by some 1e-9 (set_pair_constants).
+__device__ __forceinline__ void lj2(f32x2 r2, f32x2 cs, f32x2 c1, f32x2 c3, f32x2& fs, f32x2& q,
+                                    f32x2& q2) {
   const f32x2 s = mul2(pack2(rcp_approx(lo2(r2)), rcp_approx(hi2(r2))), cs);
-  const f32x2 s2 = mul2(s, s);
-  q = mul2(mul2(s2, s), c3);
-  const f32x2 s4 = mul2(s2, s2);
-  fs = fma2(q, s4, s4);
+  const f32x2 s2 = mul2(s, s), s3 = mul2(s2, s);
+  const f32x2 u = fma2(s3, c3, c1);
+  fs = mul2(mul2(s2, s2), u);
+  q = mul2(s3, c3);
+  q2 = add2(u, c1);
 }
 
 __device__ __forceinline__ f32x2 len2(f32x2 dx, f32x2 dy, f32x2 dz) {
@@ -216,8 +218,8 @@ __device__ __forceinline__ f32x2 len2(f32x2 dx, f32x2 dy, f32x2 dz) {
 // Atom i against two list entries j, k.  TAIL: only the first `real` of them
 // count (list padding, which may be the atom itself).
 template <bool ENERGY, bool TAIL>
-__device__ __forceinline__ void mixed_pair2(const Hi3& pi, uint4 pj, uint4 pk, f32x2 cs, f32x2 c3, f32x2 nhi,
-                                            int real, PairAcc& a) {
+__device__ __forceinline__ void mixed_pair2(const Hi3& pi, uint4 pj, uint4 pk, f32x2 cs, f32x2 c1, f32x2 c3,
+                                            f32x2 nhi, int real, PairAcc& a) {
   const f32x2 dx = pack2((float)(int)(pj.x - pi.x), (float)(int)(pk.x - pi.x));
   const f32x2 dy = pack2((float)(int)(pj.y - pi.y), (float)(int)(pk.y - pi.y));
   const f32x2 dz = pack2((float)(int)(pj.z - pi.z), (float)(int)(pk.z - pi.z));
@@ -225,20 +227,20 @@ __device__ __forceinline__ void mixed_pair2(const Hi3& pi, uint4 pj, uint4 pk, f
   const f32x2 t = add2(r2, nhi);  // negative: inside (the sign is exact)
   a.tmin = min3_abs(lo2(t), hi2(t), a.tmin);
   const f32x2 m = pack2(__saturatef(lo2(t) * -1e30f), __saturatef(hi2(t) * -1e30f));
-  f32x2 q, fs;
-  lj2(r2, cs, c3, q, fs);
-  fs = mul2(fs, m);
+  f32x2 fs, q, q2;
+  lj2(r2, mul2(cs, m), c1, c3, fs, q, q2);
   if (TAIL) fs = pack2(real > 0 ? lo2(fs) : 0.0f, real > 1 ? hi2(fs) : 0.0f);
   a.fx = fma2(fs, dx, a.fx);
   a.fy = fma2(fs, dy, a.fy);
   a.fz = fma2(fs, dz, a.fz);
   if (ENERGY) {
-    f32x2 e = mul2(fma2(q, q, add2(q, q)), m), n = m;
+    f32x2 n = m;
     if (TAIL) {
-      e = pack2(real > 0 ? lo2(e) : 0.0f, real > 1 ? hi2(e) : 0.0f);
+      q = pack2(real > 0 ? lo2(q) : 0.0f, real > 1 ? hi2(q) : 0.0f);
+      q2 = pack2(real > 0 ? lo2(q2) : 0.0f, real > 1 ? hi2(q2) : 0.0f);
       n = pack2(real > 0 ? lo2(n) : 0.0f, real > 1 ? hi2(n) : 0.0f);
     }
-    a.e = add2(a.e, e);
+    a.e = fma2(q, q2, a.e);
     a.n = add2(a.n, n);
   }
 }
@@ -247,15 +249,15 @@ __device__ __forceinline__ void mixed_pair2(const Hi3& pi, uint4 pj, uint4 pk, f
 template <bool ENERGY>
 __device__ __forceinline__ void mixed_pair_remove(float dx, float dy, float dz, float r2,
                                                   const StepConst& K, PairAcc& a) {
-  f32x2 q, fs;
-  lj2(pack2(r2, r2), pack2(K.cs, K.cs), pack2(K.c3, K.c3), q, fs);
+  f32x2 fs, q, q2;
+  lj2(pack2(r2, r2), pack2(K.cs, K.cs), pack2(K.c1, K.c1), pack2(K.c3, K.c3), fs, q, q2);
   const f32x2 m = pack2(-1.0f, 0.0f);
   fs = mul2(fs, m);
   a.fx = fma2(fs, pack2(dx, dx), a.fx);
   a.fy = fma2(fs, pack2(dy, dy), a.fy);
   a.fz = fma2(fs, pack2(dz, dz), a.fz);
   if (ENERGY) {
-    a.e = fma2(fma2(q, q, add2(q, q)), m, a.e);
+    a.e = fma2(mul2(q, m), q2, a.e);
     a.n = add2(a.n, m);
   }
 }
@@ -790,7 +792,7 @@ __device__ __forceinline__ PairAcc mixed_sublist_forces(Hi3 pi, const uint4* pos
                                                         uint32_t col, uint32_t ncols, int cnt,
                                                         const StepConst& K) {
   PairAcc a{0ull, 0ull, 0ull, 0ull, 0ull, 3.0e38f};
-  const f32x2 cs = pack2(K.cs, K.cs), c3 = pack2(K.c3, K.c3);
+  const f32x2 cs = pack2(K.cs, K.cs), c1 = pack2(K.c1, K.c1), c3 = pack2(K.c3, K.c3);
   const f32x2 nhi = pack2(-K.rc2u_hi, -K.rc2u_hi);
   const uint2* list = reinterpret_cast<const uint2*>(nb) + col;
   const int nblk = (cnt + 3) >> 2;
@@ -802,16 +804,16 @@ __device__ __forceinline__ PairAcc mixed_sublist_forces(Hi3 pi, const uint4* pos
     const uint2 wn = kb + 1 < nblk ? *list : w;
     const uint4 p0 = pos[w.x & 0xFFFFu], p1 = pos[w.x >> 16];
     const uint4 p2 = pos[w.y & 0xFFFFu], p3 = pos[w.y >> 16];
-    mixed_pair2<ENERGY, false>(pi, p0, p1, cs, c3, nhi, 2, a);
-    mixed_pair2<ENERGY, false>(pi, p2, p3, cs, c3, nhi, 2, a);
+    mixed_pair2<ENERGY, false>(pi, p0, p1, cs, c1, c3, nhi, 2, a);
+    mixed_pair2<ENERGY, false>(pi, p2, p3, cs, c1, c3, nhi, 2, a);
     w = wn;
   }
   if (nblk > nfull) {  // the last block, in part padding
     const int left = cnt & 3;
     const uint4 p0 = pos[w.x & 0xFFFFu], p1 = pos[w.x >> 16];
-    mixed_pair2<ENERGY, true>(pi, p0, p1, cs, c3, nhi, left, a);
+    mixed_pair2<ENERGY, true>(pi, p0, p1, cs, c1, c3, nhi, left, a);
     const uint4 p2 = pos[w.y & 0xFFFFu];
-    mixed_pair2<ENERGY, true>(pi, p2, p2, cs, c3, nhi, left - 2, a);
+    mixed_pair2<ENERGY, true>(pi, p2, p2, cs, c1, c3, nhi, left - 2, a);
   }
   return a;
 }
