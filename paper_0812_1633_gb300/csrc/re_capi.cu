@@ -676,7 +676,7 @@ int launch_advance(re_ctx* c, const int32_t* d_budget, const int32_t* h_budget,
       RE_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0), "fork");
       cudaError_t e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work2 + nn, nw, d_budget,
                                          fp64, wk, c->max_n, list_elems_for(c, wk),
-                                         0, c->side, nullptr);
+                                         0, c->side, nullptr, uneven);
       if (e != cudaSuccess) return cuda_fail(c, e, "batched MD launch (wide class)");
       e = re::launch_batched(c->s, c->d_ens, c->d_rep, c->d_work2, nn, d_budget, fp64, c->cfg,
                              c->max_n, list_elems_for(c, c->cfg), 0, c->stream,
