@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(512) direct_force_kernel(DirectScratch s, int 
       if (close && r2 == 0.0f && j != i) st = kStNumeric;  // at one point: no direction
       const bool hit = r2 < K.rc2u_hi && j != i;
       const uint32_t b = __ballot_sync(0xffffffffu, hit);
-      if (hit) note[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(j | (r2 > K.rc2u_lo ? 0x8000 : 0));
+      if (hit) note[n + __popc(b & ((1u << lane) - 1u))] = (uint16_t)(j | (fp64_edge(r2, K) ? 0x8000 : 0));
       n += __popc(b);
       if (n >= 32) {
         __syncwarp();

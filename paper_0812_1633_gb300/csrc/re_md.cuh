@@ -867,9 +867,15 @@ __device__ __forceinline__ double float_to_double_2m64(float v) {
 // FP64 force of one pair, separation d (units of L / 2^64), hi the FP32 r^2 of
 // its top words: 17 FP64 operations.  1/r^2 starts from the FP32 value x0 with
 // one third-order step x = x0 (1 + e + e^2), e = 1 - r^2 x0 (the partial sum
-// of the geometric series of 1 / (1 - e)), |e| < 1e-6.  All stay in units of
-// the separation: s = 1/r^2 is about 1e-37 and s^7 about 1e-260, in range.
-// edge: decided on the FP64 r^2.
+// of the geometric series of 1 / (1 - e)); |e| < 4e-6 while the top words tell the
+// atoms 2^20 units (2.4e-4 L) and more apart.  All stay in units of the separation:
+// s = 1/r^2 is about 1e-37 and s^7 about 1e-260, in range.
+// edge (fp64_edge of the top words' r^2): near the cutoff, decided on the FP64 r^2,
+// or closer than that, x0 from the FP64 r^2 (no liquid has such pairs; a test in
+// every pair took 6 % of a step).
+__device__ __forceinline__ bool fp64_edge(float r2, const StepConst& K) {
+  return r2 > K.rc2u_lo || r2 < 0x1p40f;
+}
 struct Fp64Acc {
   double fx, fy, fz, e;  // sums of 24 s^4 (1 - 2 s^3) d and of the pair energies
 };
@@ -882,9 +888,12 @@ __device__ __forceinline__ void fp64_pair(const Pos64& pi, const Pos64& pj, cons
   const double dx = (double)(long long)(pj.x - pi.x), dy = (double)(long long)(pj.y - pi.y),
                dz = (double)(long long)(pj.z - pi.z);
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  if (edge && !(r2 < c.rc2)) return;
-  const double x0 = float_to_double_2m64(
+  double x0 = float_to_double_2m64(
       rcp_approx(sep2_hi(hi, Hi3{(uint32_t)(pj.x >> 32), (uint32_t)(pj.y >> 32), (uint32_t)(pj.z >> 32)})));
+  if (edge) {
+    if (!(r2 < c.rc2)) return;
+    if (r2 < 0x1p105) x0 = (double)rcp_approx((float)r2);
+  }
   const double er = fma(-r2, x0, 1.0);
   const double s = fma(x0, fma(er, er, er), x0);
   const double s2 = s * s, s3 = s2 * s;
@@ -908,8 +917,8 @@ __device__ __forceinline__ void fp64_pair(const Pos64& pi, const Pos64& pj, cons
 // dealt out evenly (buf: 32 noted entries a thread in shared memory), since
 // one lane's 14 +- 3 hits would make the fullest of 32 lanes need 21 to 24
 // turns; with fewer lanes each goes through its own hits (a bit mask), 28 +- 4
-// or 55 +- 5 of them.  Entries within 2e-6 of rc^2 are decided on the FP64
-// r^2.
+// or 55 +- 5 of them.  Entries within 2e-6 of rc^2, and very close ones, are
+// marked (fp64_edge).
 template <bool ENERGY, int P>
 __device__ __forceinline__ Fp64Acc fp64_sublist_forces(const Pos64* pos, int i, bool own,
                                                        const uint16_t* __restrict__ nb, uint32_t col,
@@ -938,7 +947,7 @@ __device__ __forceinline__ Fp64Acc fp64_sublist_forces(const Pos64* pos, int i, 
       for (int k = 0; k < 4; ++k) {
         const uint32_t j = ((k < 2 ? w.x : w.y) >> (16 * (k & 1))) & 0xFFFFu;
         const float r2 = sep2_hi(hi, hi_of((int)j));
-        const bool hit = k0 + b + k < cnt && r2 < K.rc2u_hi, edge = r2 > K.rc2u_lo;
+        const bool hit = k0 + b + k < cnt && r2 < K.rc2u_hi, edge = fp64_edge(r2, K);
         if (P >= 4) {
           if (hit) mine[n++] = (uint16_t)(j | (edge ? 0x8000u : 0u));
         } else if (hit) {
