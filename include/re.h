@@ -364,7 +364,8 @@ int re_exchange_device_h(int R, const double *T, const double *lam, const double
  * (AoS), f device array of 3N doubles, U device pointer to one double.
  * precision: RE_PREC_FP64 or RE_PREC_MIXED, with the pair arithmetic of the MD
  * path; the replica sizes and, within rc + 0.5 of an atom, the neighbours that
- * its default lists hold are the limits (RE_EINVAL, RE_EOVERFLOW beyond).
+ * its default lists hold are the limits (RE_EINVAL, RE_EOVERFLOW beyond).  A call
+ * that fails leaves f and U as they were.  f may be x.
  * Scratch comes from a memory pool of the library's own, stream-ordered, and
  * goes back before return; the call synchronises `stream`.  Calls from several
  * threads and streams do not affect one another.  Requires 2 <= N <= 65535 and
@@ -377,7 +378,7 @@ int re_lj_forces_device(int N, double L, double rc, int shift, int precision, co
  * another framework's memory pool or under a fixed memory budget, plug-ins
  * that may not touch the allocator).  The paper has no counterpart: this is a
  * deployment variant.  Scratch lives in one fixed device array of about
- * 140 KB that every device loading the library keeps until the process exits.
+ * 240 KB that every device loading the library keeps until the process exits.
  * Limits: 2 <= N <= 4096 atoms, at most 256 neighbours within rc + 0.5 per atom
  * (RE_EOVERFLOW beyond), rc + 0.5 < L/2.  Arguments as re_lj_forces_device
  * (device pointers, caller-owned).  The first call on a device looks up the

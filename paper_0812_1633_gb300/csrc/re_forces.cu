@@ -5,8 +5,9 @@
 namespace re {
 namespace {
 
-// Fixed-point words of the caller's positions; clears the words of the call.
-__global__ void __launch_bounds__(256) direct_fix_kernel(const double* __restrict__ x, DirectScratch s,
+// Fixed-point words of the caller's positions; clears the words of the call and
+// keeps what f holds (which may be x): a call that fails gives it back.
+__global__ void __launch_bounds__(256) direct_fix_kernel(const double* x, const double* f, DirectScratch s,
                                                          int N, double inv_l) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) {
@@ -16,6 +17,7 @@ __global__ void __launch_bounds__(256) direct_fix_kernel(const double* __restric
     s.hi[i] = make_uint4((uint32_t)(q[0] >> 32), (uint32_t)(q[1] >> 32), (uint32_t)(q[2] >> 32), 0u);
     s.lo[i] = make_uint4((uint32_t)q[0], (uint32_t)q[1], (uint32_t)q[2], 0u);
   }
+  for (int k = i; k < 3 * N; k += gridDim.x * blockDim.x) s.old[k] = f[k];
   if (i < 2) s.words[i] = 0;
 }
 
@@ -135,14 +137,17 @@ __global__ void __launch_bounds__(512) direct_force_kernel(DirectScratch s, int 
       __threadfence();
       last = atomicAdd(s.words, 1) == (int)gridDim.x - 1;
     }
-    __syncwarp();
-    if (last) {
-      __threadfence();
-      double u = 0.0;
-      for (int b = lane; b < (int)gridDim.x; b += 32) u += __ldcg(s.part + b);
-      u = warp_sum(u);
-      if (lane == 0) *U = 0.5 * u;
-    }
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (__ldcg(s.words + 1) != 0) {  // failed: f and U stay as they were
+    for (int k = threadIdx.x; k < 3 * N; k += blockDim.x) f[k] = s.old[k];
+  } else if (warp == 0) {
+    double u = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) u += __ldcg(s.part + b);
+    u = warp_sum(u);
+    if (lane == 0) *U = 0.5 * u;
   }
 }
 
@@ -153,7 +158,7 @@ int direct_warps(int N, int sms) { return std::min(16, std::max(4, (N + 2 * sms 
 }  // namespace
 
 size_t direct_scratch_bytes(int N) {
-  return (size_t)N * 32 + (((size_t)N + 3) / 4 + 2) * sizeof(double);
+  return (size_t)N * (32 + 3 * sizeof(double)) + (((size_t)N + 3) / 4 + 2) * sizeof(double);
 }
 
 cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixed, int cap, int sms,
@@ -162,10 +167,11 @@ cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixe
   DirectScratch s;
   s.hi = static_cast<uint4*>(scratch);
   s.lo = s.hi + N;
-  s.part = reinterpret_cast<double*>(s.lo + N);
+  s.old = reinterpret_cast<double*>(s.lo + N);
+  s.part = s.old + 3 * (size_t)N;
   s.words = reinterpret_cast<int32_t*>(s.part + (N + 3) / 4);
   *status = s.words + 1;
-  direct_fix_kernel<<<(N + 255) / 256, 256, 0, st>>>(x, s, N, K.inv_l);
+  direct_fix_kernel<<<(N + 255) / 256, 256, 0, st>>>(x, f, s, N, K.inv_l);
   const int W = direct_warps(N, sms);
   const size_t smem = (size_t)N * 16;
   auto fn = mixed ? direct_force_kernel<true> : direct_force_kernel<false>;

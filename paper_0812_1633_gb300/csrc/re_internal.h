@@ -304,6 +304,7 @@ cudaError_t launch_spatial_sort(const StateDev& s, const EnsDev* d_ens, const Re
 // that an atom may have (beyond: kStOverflow in *status, a device word).
 struct DirectScratch {
   uint4 *hi, *lo;  // N each: top and low 32 bits of the fixed-point positions
+  double* old;     // 3N: what f held before the call
   double* part;    // energy of each CTA
   int32_t* words;  // CTAs done, status bits
 };

@@ -29,7 +29,7 @@ namespace {
 constexpr int kMaxAtoms = 4096;
 constexpr int kMaxNeighbours = 256;
 constexpr int kMaxDevices = 64;
-constexpr size_t kScratch = (size_t)kMaxAtoms * 32 + ((size_t)kMaxAtoms / 4 + 2) * 8;
+constexpr size_t kScratch = (size_t)kMaxAtoms * 56 + ((size_t)kMaxAtoms / 4 + 2) * 8;
 
 // device address of g_scratch, per device; every thread that fills an entry
 // stores the same value, so relaxed atomic accesses suffice
