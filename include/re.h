@@ -26,7 +26,8 @@
  *     that synchronises (getters, re_sync).
  *   - Threads: one host thread per context at a time.  Calls are queued on the
  *     context's CUDA stream (re_set_stream); getters synchronise that stream.
- *   - The library allocates its own device memory with cudaMalloc at creation.
+ *   - The library allocates its own device memory with cudaMalloc at creation
+ *     (re_lj_forces_device: see there).
  *
  * Random numbers: Philox4x64-10 (Salmon et al., SC'11) used as a
  * counter-based generator; key = (seed, stream), counter = (index, tag, sub, 0):
@@ -367,7 +368,9 @@ int re_exchange_device_h(int R, const double *T, const double *lam, const double
  * its default lists hold are the limits (RE_EINVAL, RE_EOVERFLOW beyond).  A call
  * that fails leaves f and U as they were.  f may be x.
  * Scratch comes from a memory pool of the library's own, stream-ordered, and
- * goes back before return; the call synchronises `stream`.  Calls from several
+ * goes back to it before return; the pool keeps up to 64 MB of device memory
+ * until the process exits or a context's allocations need it.  The call
+ * synchronises `stream`.  Calls from several
  * threads and streams do not affect one another.  Requires 2 <= N <= 65535 and
  * rc + 0.5 < L/2. */
 int re_lj_forces_device(int N, double L, double rc, int shift, int precision, const double *x,

@@ -203,11 +203,61 @@ int cuda_fail(re_ctx* c, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(c, e_, what); \
   } while (0)
 
+// The memory pools of re_lj_forces_device, one per device: stream-ordered, so
+// calls from any threads and streams share one; it keeps at most 64 MB between
+// calls (the driver's pools grow by 32 MB; keeping less than that, every call
+// maps memory anew, 220 us) and returns the rest, and that too where another
+// allocation of the library would fail for it (trim_scratch_pool).  The some 45
+// allocations of a context took half a millisecond a call and more.
+struct ScratchPools {
+  std::mutex mu;
+  cudaMemPool_t of[64] = {};
+};
+ScratchPools g_scratch_pools;
+
+cudaError_t scratch_pool(cudaMemPool_t* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(g_scratch_pools.mu);
+  cudaMemPool_t& pool = g_scratch_pools.of[dev];
+  if (!pool) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+    uint64_t keep = 64ull << 20;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    pool = p;
+  }
+  *out = pool;
+  return cudaSuccess;
+}
+
+// Gives back what the current device's pool keeps; false when it has none.
+bool trim_scratch_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  std::lock_guard<std::mutex> lock(g_scratch_pools.mu);
+  const cudaMemPool_t pool = g_scratch_pools.of[dev];
+  return pool && cudaMemPoolTrimTo(pool, 0) == cudaSuccess;
+}
+
 template <class T>
 int dalloc(re_ctx* c, T** p, size_t n) {
   void* q = nullptr;
   size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
   cudaError_t e = cudaMalloc(&q, bytes);
+  if (e == cudaErrorMemoryAllocation && trim_scratch_pool()) {
+    cudaGetLastError();
+    e = cudaMalloc(&q, bytes);
+  }
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaMalloc");
   c->allocs.push_back(q);
   *p = static_cast<T*>(q);
@@ -2253,41 +2303,6 @@ int re_exchange_device_h(int R, const double* T, const double* lam, const double
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "exchange launch");
   return RE_OK;
 }
-
-namespace {
-
-// The memory pool of re_lj_forces_device on the current device: stream-ordered,
-// so calls from any threads and streams share it; it keeps at most 64 MB between
-// calls (the driver's pools grow by 32 MB; keeping less than that, every call
-// maps memory anew, 220 us) and returns the rest.  The some 45 allocations of a
-// context took half a millisecond a call and more.
-cudaError_t scratch_pool(cudaMemPool_t* out) {
-  static std::mutex mu;
-  static cudaMemPool_t pools[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(mu);
-  if (!pools[dev]) {
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t p = nullptr;
-    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
-    uint64_t keep = 64ull << 20;
-    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
-      cudaMemPoolDestroy(p);
-      return e;
-    }
-    pools[dev] = p;
-  }
-  *out = pools[dev];
-  return cudaSuccess;
-}
-
-}  // namespace
 
 int re_lj_forces_device(int N, double L, double rc, int shift, int precision, const double* x,
                         double* f, double* U, void* stream) {
