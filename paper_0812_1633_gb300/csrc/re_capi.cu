@@ -576,6 +576,9 @@ int check_cfg(re_ctx* c, const LaunchCfg& k, const Scope& sc) {
       k.threads < k.atom_threads * ((sc.max_n + k.cluster - 1) / k.cluster))
     return fail(c, RE_EINVAL, "%d atoms per CTA x %d threads per atom exceed 1024 threads; "
                 "use more CTAs per replica", (sc.max_n + k.cluster - 1) / k.cluster, k.atom_threads);
+  if (sc.max_n > re::kMaxBatchedAtoms)
+    return fail(c, RE_EINVAL, "replica of %d atoms: the batched path takes at most %d", sc.max_n,
+                re::kMaxBatchedAtoms);
   const size_t smem = re::batched_admission_bytes(sc.max_n, sc.max_ncell, k.threads,
                                                   c->opt.precision == RE_PREC_FP64) +
                       re::kBatchedStaticSmem;

@@ -164,6 +164,7 @@ size_t direct_scratch_bytes(int N) {
 cudaError_t launch_lj_direct(void* scratch, int N, const StepConst& K, bool mixed, int cap, int sms,
                              const double* x, double* f, double* U, int32_t** status,
                              cudaStream_t st) {
+  if (N > kMaxNotedAtoms) return cudaErrorInvalidValue;
   DirectScratch s;
   s.hi = static_cast<uint4*>(scratch);
   s.lo = s.hi + N;

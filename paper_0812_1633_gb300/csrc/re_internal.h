@@ -129,6 +129,15 @@ struct RepDev {
 // by testing every atom, larger ones by screening (re_md.cuh).
 constexpr int kDirectBuild = 256;
 
+// The most atoms of a replica on the batched path: the screened build keeps the
+// numbers of its rows of 32 atoms in bytes.  (Shared memory admits some 6800,
+// batched_admission_bytes.)
+constexpr int kMaxBatchedAtoms = 256 * 32;
+// The most atoms of a direct force call, and of the FP64 pair loop: noted atoms are
+// 15-bit numbers and a flag.
+constexpr int kMaxNotedAtoms = 1 << 15;
+static_assert(kMaxBatchedAtoms <= kMaxNotedAtoms, "the FP64 pair loop notes any atom of a replica");
+
 // Notes (candidate masks, 8 bytes each) that the screened list build of a lane
 // can keep in the part of its replica's list array that a layout of P threads per
 // atom leaves unused (the array holds the largest layout, P = 8).
@@ -300,8 +309,9 @@ cudaError_t launch_spatial_sort(const StateDev& s, const EnsDev* d_ens, const Re
                                 cudaStream_t st);
 // Forces and energy of one configuration (re_forces.cu): positions, partial sums
 // and words of a call in one scratch area of direct_scratch_bytes(N) bytes,
-// 16-byte aligned; N <= 32767.  cap: neighbours within the list radius of K
-// that an atom may have (beyond: kStOverflow in *status, a device word).
+// 16-byte aligned; N <= kMaxNotedAtoms (cudaErrorInvalidValue beyond).  cap:
+// neighbours within the list radius of K that an atom may have (beyond:
+// kStOverflow in *status, a device word).
 struct DirectScratch {
   uint4 *hi, *lo;  // N each: top and low 32 bits of the fixed-point positions
   double* old;     // 3N: what f held before the call

@@ -1057,6 +1057,7 @@ cudaError_t launch_batched(const StateDev& s, const EnsDev* d_ens, const RepDev*
                            const LaunchCfg& cfg, int max_n, size_t list_elems,
                            int async_nx, cudaStream_t st, const FreeDev* fr, bool uneven) {
   if (n_work <= 0) return cudaSuccess;
+  if (max_n > kMaxBatchedAtoms) return cudaErrorInvalidValue;
   const bool lsm = list_elems > 0;
   const int mode = (fr && fr->nx > 0) ? 2 : (async_nx > 0 ? 1 : 0);
   // the two free-running modes keep the lists in global memory
