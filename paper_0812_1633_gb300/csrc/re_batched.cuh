@@ -28,8 +28,8 @@ namespace {
 // MODE 0: per-replica step budgets; 1: master-stop (dims.async_nx); 2:
 // free-running with exchanges inside the launch (fr).
 // MAXT: the most threads per CTA of this instantiation; it sets the register
-// budget (1024: 64 registers per thread; kNarrowThreads = 896: 72), and the
-// launcher picks the narrowest instantiation that holds the launch's CTAs.
+// budget (1024: 64 registers per thread; kNarrowThreads = 896: 72).  CTAs of up to
+// kNarrowThreads threads run in either; narrow_build chooses.
 template <bool FP64, int P, bool LSM, int MODE, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
                                                              const EnsDev* __restrict__ ens,
@@ -272,10 +272,12 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   int nreb = 0;
   // Rebuild of the lists of this CTA's atoms.
   auto rebuild = [&]() {
-    if (N <= kDirectBuild * P) {
+    bool direct = true;  // eight threads an atom: at most 1024 atoms
+    if constexpr (P <= 4) direct = N <= kDirectBuild * P;
+    if (direct) {
       cnt = build_sublist_direct<P>(i, q, own, hi_of, N, K.rl2u, nb, mycol, ncols, cap_sub,
                                     &overflow);
-    } else {
+    } else if constexpr (P <= 4) {
       cta_screen_vectors(hi_of, N, sm.hk, sm.box);
       cnt = build_sublist<P>(i, own, i0 + warp * (32 / P), hi_of, N, sm.hk, sm.box,
                              sm.act + warp * row_list_bytes(N), K.rl2u, nb, mycol, ncols,

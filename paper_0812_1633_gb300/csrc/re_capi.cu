@@ -280,7 +280,6 @@ void finish_ens(EnsDev& e) {
   k.uc = e.shift ? 4.0 * (1.0 / (rc6 * rc6) - 1.0 / rc6) : 0.0;
   k.rc2 = e.rc * e.rc;
   const double rcu = e.rc / k.lam32;
-  k.rc2u = (float)(rcu * rcu);
   k.rc2u_lo = (float)(rcu * rcu * (1.0 - 2e-6));
   k.rc2u_hi = (float)(rcu * rcu * (1.0 + 2e-6));
   const double rcx = e.rc / (e.L * 0x1.0p-42);
@@ -296,7 +295,6 @@ void finish_ens(EnsDev& e) {
   const double omc = e.tau > 0.0 ? -std::expm1(-e.dt / e.tau) : 0.0;  // 1 - c, no cancellation
   k.cm1f = (float)(-omc);
   // Kbar = Nf T / 2: a = (1 - c) T / 2, b = 2 sqrt(c (1 - c) T / 2), g = sqrt(2 c / ((1 - c) T))
-  k.kbar1 = 0.5 * k.nf;
   k.af1 = 0.5 * omc;
   k.bf1 = 2.0 * std::sqrt(0.5 * k.c_th * omc);
   k.gf1 = omc > 0.0 ? std::sqrt(2.0 * k.c_th / omc) : 0.0;

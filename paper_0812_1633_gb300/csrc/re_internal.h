@@ -35,20 +35,21 @@ enum StatusBits : int {
 
 // Per-ensemble step constants, formed once on the host (FP64 transcendentals
 // and divisions run at 1/64 of the FP32 rate on the GPU).  The fields that
-// depend on the thermostat's target T (kbar, af, bf, gf) are filled per
-// replica by set_thermo_target.
+// depend on the thermostat's target T (af, bf, gf) are filled per replica by
+// set_thermo_target.
 struct StepConst {
-  double lam32, lam64, inv_l, dtq, hdt, inv_hdt, uc, rc2, c_th, kbar;
-  double kbar1, af1, bf1, gf1;  // kbar = kbar1 T, af = af1 T, bf = bf1 sqrt(T), gf = gf1 / sqrt(T)
+  double lam32, lam64, inv_l, dtq, hdt, inv_hdt, uc, rc2, c_th;
+  double af1, bf1, gf1;         // af = af1 T, bf = bf1 sqrt(T), gf = gf1 / sqrt(T)
   double lamv;                  // the replica's potential scale (set_potential_scale)
   double f24;                   // 24 kappa^4 / c1
   double rc2x;                  // rc^2 in units (L / 2^42)^2 (exact cutoff test, mixed path)
   float hlf;                    // FP32 half-kick factor per unit of the mixed pair sums, times lamv
-  float rc2u, rl2u, half2u;
+  float rl2u, half2u;
   // mixed pair sums (set_pair_constants), (2^32 / L)^2 = kappa 2^k: cs = -2^k,
   // c3 / c1 = 2 kappa^3, eu + eul = 1 / c1^2
   float cs, c1, c3, eu, eul;
-  float rc2u_lo, rc2u_hi;       // rc2u (1 -+ 2e-6): the band decided on 42-bit separations
+  float rc2u_lo, rc2u_hi;       // rc^2 (1 -+ 2e-6), units (L / 2^32)^2: the band decided on
+                                // 42-bit separations
   // thermostat constants of the mixed path (used in FP32): c - 1,
   // (1 - c) Kbar / Nf, 2 sqrt(c (1 - c) Kbar / Nf), sqrt(c Nf / ((1 - c) Kbar))
   float cm1f, af, bf, gf;
@@ -112,7 +113,6 @@ __host__ __device__ inline void set_potential_scale(StepConst& k, double lam) {
 
 // The constants of StepConst that depend on the target temperature T.
 __host__ __device__ inline void set_thermo_target(StepConst& k, double T) {
-  k.kbar = k.kbar1 * T;
   k.af = (float)(k.af1 * T);
   const float ts = sqrtf((float)T);
   k.bf = (float)k.bf1 * ts;
@@ -153,7 +153,7 @@ struct StateDev {
   uint16_t* nbr;
   uint16_t* raw;  // as nbr: notes of the list builds, where list_notes() finds no room (else null)
   double *T, *U, *K, *econs, *vscale;
-  double *lam, *fscale;  // per replica: potential scale; pending force factor (null: 1)
+  double *lam, *fscale;  // per replica: potential scale; pending force factor
   int64_t *step, *nreb;
   int32_t *status, *valid;
   int64_t* attempt;                  // per ensemble

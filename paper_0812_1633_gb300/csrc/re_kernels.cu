@@ -7,9 +7,10 @@
 //   md_batched_kernel  one thread-block cluster per replica runs that
 //                      replica's whole step budget: kick, drift, displacement
 //                      test, [list build: candidates screened on the tensor
-//                      cores, exact integer test], LJ forces, kick, thermostat.  Positions of the replica
-//                      live in shared memory of every CTA of the cluster
-//                      (broadcast through distributed shared memory).
+//                      cores, exact integer test], LJ forces, kick, thermostat.
+//                      Positions of the replica live in shared memory of every
+//                      CTA of the cluster (broadcast through distributed shared
+//                      memory).
 //   plain_*            the same step as a sequence of launches for one
 //                      replica at a time, FP64 throughout (comparison path).
 //   exchange_kernel    Implementation section: sort temperatures, pair
@@ -121,7 +122,7 @@ __global__ void plain_kick_drift(StateDev S, const EnsDev* __restrict__ ens,
   const EnsDev E = ens[rd.ens];
   const StepConst& K = E.kc;
   const double vs = S.vscale[r];
-  const double fs = S.fscale ? S.fscale[r] : 1.0;  // pending force factor (exchange of lam)
+  const double fs = S.fscale[r];  // pending force factor (exchange of lam)
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float md = 0.0f;
   if (i < E.N) {
@@ -180,8 +181,7 @@ __global__ void plain_rebuild(StateDev S, const EnsDev* __restrict__ ens,
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int g = rd.atom_off + i;
     S.ncnt[(size_t)rd.atom_off * 8 + i] =
-        build_sublist_cells<1>(i, 0, hi_of, N, E.nc, E.m, cstart, spos, K.rl2u, nb, (uint32_t)i,
-                         (uint32_t)N, E.capsub[0], &overflow);
+        build_list_cells(i, hi_of, N, E.nc, E.m, cstart, spos, K.rl2u, nb, E.capsub[0], &overflow);
     S.rx[g] = hp[i].x;
     S.ry[g] = hp[i].y;
     S.rz[g] = hp[i].z;
@@ -228,7 +228,7 @@ __global__ void plain_forces(StateDev S, const EnsDev* __restrict__ ens,
         e += 4.0 * (s3 * s3 - s3) - K.uc;
       }
     }
-    const double lam = S.lam ? S.lam[r] : 1.0;
+    const double lam = S.lam[r];
     S.fx[g] = lam * fx;
     S.fy[g] = lam * fy;
     S.fz[g] = lam * fz;
@@ -718,7 +718,7 @@ __global__ void apply_vscale_kernel(StateDev S, const RepDev* __restrict__ reps,
   const RepDev rd = reps[r];
   const int N = ens[rd.ens].N;
   const double vs = S.vscale[r];
-  const double fs = S.fscale ? S.fscale[r] : 1.0;
+  const double fs = S.fscale[r];
   if (vs == 1.0 && fs == 1.0) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const int g = rd.atom_off + i;
@@ -806,8 +806,8 @@ __global__ void import_kernel(StateDev S, const EnsDev* __restrict__ ens,
   const double inv_l = 1.0 / E.L;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < E.N; i += gridDim.x * blockDim.x) {
     const int g = rd.atom_off + i;
-    // original order (no permutation array: slots are the original order)
-    const size_t o = (size_t)rd.atom_off + (S.perm ? S.perm[g] : i);
+    // original order
+    const size_t o = (size_t)rd.atom_off + S.perm[g];
     if (x) {
       S.qx[g] = fix_from_double(x[3 * o + 0], inv_l);
       S.qy[g] = fix_from_double(x[3 * o + 1], inv_l);
@@ -1188,7 +1188,7 @@ cudaError_t launch_import_state(const StateDev& s, const EnsDev* d_ens, const Re
 
 cudaError_t launch_identity_perm(const StateDev& s, const EnsDev* d_ens, const RepDev* d_rep,
                                  int n_rep, cudaStream_t st) {
-  if (n_rep <= 0 || !s.perm) return cudaSuccess;
+  if (n_rep <= 0) return cudaSuccess;
   identity_perm_kernel<<<dim3(16, n_rep), 256, 0, st>>>(s, d_ens, d_rep);
   return cudaGetLastError();
 }

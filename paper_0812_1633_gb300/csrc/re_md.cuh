@@ -353,19 +353,16 @@ __device__ __forceinline__ uint32_t* rcomp(const StateDev& S, int d) {
   return d == 0 ? S.rx : (d == 1 ? S.ry : S.rz);
 }
 
-// Sub-list of lane q (of P) of atom i: candidates of every scanned range are
-// dealt to the P lanes in turn (candidate k of a range goes to lane k % P).
-// Entry k of sub-list (i, q) sits at nb[((k/4) * N*P + i*P + q) * 4 + k%4].
-// The sub-list of column `col` of a list with `ncols` columns: entry k at
-// element ((k / 4) * ncols + col) * 4 + k % 4 of nb.
-template <int P, class PosFn>
-__device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, int m, const int* cstart,
-                             const uint4* spos, float rl2u, uint16_t* nb, uint32_t col,
-                             uint32_t ncols, int cap_sub, int* overflow) {
+// The list of atom i on the plain path (one thread an atom), from the cells
+// (nc > 0) or all atoms: entry k at element ((k / 4) * N + i) * 4 + k % 4 of nb.
+template <class PosFn>
+__device__ int build_list_cells(int i, PosFn pos_hi, int N, int nc, int m, const int* cstart,
+                                const uint4* spos, float rl2u, uint16_t* nb, int cap,
+                                int* overflow) {
   const Hi3 pi = pos_hi(i);
-  // a running offset: +1 inside a block of four, + ncols*4 - 3 across blocks
-  uint32_t wofs = col * 4;
-  const uint32_t jump = ncols * 4 - 3u;
+  // a running offset: +1 inside a block of four, + N*4 - 3 across blocks
+  uint32_t wofs = (uint32_t)i * 4;
+  const uint32_t jump = (uint32_t)N * 4 - 3u;
   int cnt = 0;
   bool coincident = false;
   auto accept = [&](int j, Hi3 pj) {
@@ -374,7 +371,7 @@ __device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, in
       // two distinct atoms at one point (closer than L / 2^32): the pair loop
       // treats distance 0 as the sub-list padding, so report it (below)
       coincident |= (r2 == 0.0f);
-      if (cnt < cap_sub) {
+      if (cnt < cap) {
         nb[wofs] = (uint16_t)j;
         wofs += ((cnt & 3) == 3) ? jump : 1u;
       }
@@ -382,7 +379,7 @@ __device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, in
     }
   };
   if (nc == 0) {
-    for (int j = q; j < N; j += P) accept(j, pos_hi(j));
+    for (int j = 0; j < N; ++j) accept(j, pos_hi(j));
   } else {
     const int cx = (int)__umulhi(pi.x, (uint32_t)nc), cy = (int)__umulhi(pi.y, (uint32_t)nc),
               cz = (int)__umulhi(pi.z, (uint32_t)nc);
@@ -409,9 +406,9 @@ __device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, in
         const int n1 = e1 - b1, n = n1 + (e2 - b2);
         // two candidates per iteration: both loads issue before either test
         // (four were measured slower)
-        int t = q;
-        for (; t + P < n; t += 2 * P) {
-          const int t2 = t + P;
+        int t = 0;
+        for (; t + 1 < n; t += 2) {
+          const int t2 = t + 1;
           const uint4 v = spos[t < n1 ? b1 + t : b2 + (t - n1)];
           const uint4 w = spos[t2 < n1 ? b1 + t2 : b2 + (t2 - n1)];
           accept((int)v.w, Hi3{v.x, v.y, v.z});
@@ -425,9 +422,9 @@ __device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, in
     }
   }
   if (coincident) *overflow |= kStNumeric;
-  if (cnt > cap_sub) {
+  if (cnt > cap) {
     *overflow |= kStOverflow;
-    cnt = cap_sub;
+    cnt = cap;
   }
   // pad to a whole block of four with the atom's own index (skipped by r2 > 0)
   for (int k = cnt; k & 3; ++k) nb[wofs++] = (uint16_t)i;
@@ -442,8 +439,8 @@ __device__ int build_sublist_cells(int i, int q, PosFn pos_hi, int N, int nc, in
 // distance r it is at least 3 cos(a r / sqrt 3) (cos(a sqrt u) is convex in u,
 // so the least sum at a given r^2 is the one of equal components).  One
 // mma.m16n8k8 (f16 vectors, f32 sums; the other two of its eight products add
-// the limit, and put the last row's missing atoms beyond it) screens 16 atoms against 8; one funnel shift per result collects
-// its sign.  Of the candidates that pass (7 to 20 % more than the list at
+// the limit, and put the last row's missing atoms beyond it) screens 16 atoms
+// against 8; one funnel shift per result collects its sign.  Of the candidates that pass (7 to 20 % more than the list at
 // L = 17 to 10) the exact test on the 32-bit positions keeps the list, so the
 // pair set does not depend on the screening.  No cells are built or sorted: a
 // warp goes through the rows (32 consecutive atoms) whose bounding box lies
@@ -613,6 +610,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
                                              uint32_t ncols, uint16_t* raw, uint32_t rcol,
                                              uint32_t rncols, int max_notes, int cap_sub,
                                              int* status) {
+  static_assert(P <= 4, "eight threads an atom: build_sublist_direct");
   const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
   if (!__any_sync(0xffffffffu, own)) return 0;
   const Hi3 pi = own ? pos_hi(i) : Hi3{0u, 0u, 0u};
@@ -658,7 +656,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
     for (int k = 0; k < NT; ++k)
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int a = P == 1 ? 4 * g + 2 * k + u : (P == 2 ? 2 * g + u : (P == 4 ? g : g >> 1));
+        const int a = P == 1 ? 4 * g + 2 * k + u : (P == 2 ? 2 * g + u : g);
         A[k][u] = t == 3 ? lim2 : h[min(iw + a, N - 1) * 4 + t] ^ 0x80008000u;
       }
   }
@@ -762,7 +760,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
       mk[0] = __byte_perm(c0, c1, 0x3726);
       mk[NM - 1] = __byte_perm(c0, c1, 0x1504);
     } else {
-      mk[0] = (P == 4 ? m[0] : m[0] & (g & 1 ? 0x33333333u : 0xCCCCCCCCu)) & valid;
+      mk[0] = m[0] & valid;
     }
     const uint32_t rows4 = *reinterpret_cast<const uint32_t*>(act + a0);
 #pragma unroll 1
@@ -779,8 +777,7 @@ __device__ __forceinline__ int build_sublist(int i, bool own, int iw, PosFn pos_
   drain();
   if (!own) return 0;
   // of the atom's lanes, the one whose columns hold the atom met it once
-  const bool self = P == 1 || (P == 2 && (t & 1) == (i & 1)) || (P == 4 && t == (i & 3)) ||
-                    (P == 8 && t == (i & 3) && (g & 1) == ((i >> 3) & 1));
+  const bool self = P == 1 || (P == 2 && (t & 1) == (i & 1)) || (P == 4 && t == (i & 3));
   return finish_sublist(cnt, blk, out, i, zeros > (self ? 1 : 0), cap_sub, status);
 }
 
