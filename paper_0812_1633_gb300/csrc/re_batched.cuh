@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   int nreb = 0;
   // Rebuild of the lists of this CTA's atoms.
   auto rebuild = [&]() {
-    bool direct = true;  // eight threads an atom: at most 1024 atoms
-    if constexpr (P <= 4) direct = N <= kDirectBuild * P;
+    bool direct = true;  // eight threads an atom: at most 1024 atoms, no room for notes
+    if constexpr (P <= 4) direct = N <= kDirectBuild;
     if (direct) {
       cnt = build_sublist_direct<P>(i, q, own, hi_of, N, K.rl2u, nb, mycol, ncols, cap_sub,
                                     &overflow);

@@ -432,7 +432,7 @@ bool notes_need_room(const re_ctx* c) {
   if (c->opt.path != RE_PATH_BATCHED) return false;
   for (const EnsDev& e : c->ens)
     for (int k = 0; k < 3; ++k)
-      if (e.N > (re::kDirectBuild << k) && re::list_notes(e.cap, e.capsub[k], 1 << k) < 4) return true;
+      if (e.N > re::kDirectBuild && re::list_notes(e.cap, e.capsub[k], 1 << k) < 4) return true;
   return false;
 }
 

@@ -125,9 +125,9 @@ struct RepDev {
   int64_t nbr_off;
 };
 
-// Replicas of at most this many atoms per thread of an atom have their lists built
-// by testing every atom, larger ones by screening (re_md.cuh).
-constexpr int kDirectBuild = 256;
+// Replicas of at most this many atoms have their lists built by testing every atom,
+// larger ones by screening (re_md.cuh), except with eight threads an atom.
+constexpr int kDirectBuild = 640;
 
 // The most atoms of a replica on the batched path: the screened build keeps the
 // numbers of its rows of 32 atoms in bytes.  (Shared memory admits some 6800,

@@ -556,10 +556,15 @@ __device__ __forceinline__ int deal_sublist(int i, int q, bool redo, PosFn pos_h
 }
 
 // The list of a small replica, by testing every atom: lane q takes the atoms j
-// with j % P == q, in increasing order.  Below kDirectBuild atoms a lane this
-// costs less than the screening and its notes (20 instructions an atom, no
-// divergence; re_internal.h): with P = 4 at 500 atoms 19.6 thousand clocks a build against
-// 23.5; with P = 2 at 864 atoms, past the line, 58 against 53.
+// with j % P == q, in increasing order: 20 instructions an atom, no divergence.
+// Both builds share an atom's work among its P lanes, so the line between them is
+// a number of atoms, and their cost grows with N here and with the list there.
+// Steps with a rebuild in 2.6 of them (four replicas, skin 0.1), testing every atom
+// against screening, us: 256 atoms P = 1, 2, 4 11.9, 9.0, 6.8 against 17.3, 11.5,
+// 8.3; 500 atoms P = 1, 2, 4 (eight CTAs) 15.4, 11.7, 8.6 against 21.1, 12.6, 9.5;
+// 864 atoms P = 4 on four and eight CTAs 21.9 and 15.0 against 14.2 and 11.3 (no
+// FCC box lies between).  With eight lanes screening gains at 864 atoms, 13.1
+// against 14.6, but would need room for its notes.
 template <int P, class PosFn>
 __device__ __forceinline__ int build_sublist_direct(int i, int q, bool own, PosFn pos_hi, int N,
                                                     float rl2u, uint16_t* nb, uint32_t col,
