@@ -272,8 +272,9 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
   int nreb = 0;
   // Rebuild of the lists of this CTA's atoms.
   auto rebuild = [&]() {
-    bool direct = true;  // eight threads an atom: at most 1024 atoms, no room for notes
-    if constexpr (P <= 4) direct = N <= kDirectBuild;
+    // notes of the screened build; eight threads an atom leave no room for them
+    const int notes = S.raw ? cap_sub / 4 : list_notes(E.cap, cap_sub, P);
+    const bool direct = P == 8 || N <= kDirectBuild || notes < 1;
     if (direct) {
       cnt = build_sublist_direct<P>(i, q, own, hi_of, N, K.rl2u, nb, mycol, ncols, cap_sub,
                                     &overflow);
@@ -282,8 +283,7 @@ __global__ void __launch_bounds__(MAXT, 1) md_batched_kernel(StateDev S,
       cnt = build_sublist<P>(i, own, i0 + warp * (32 / P), hi_of, N, sm.hk, sm.box,
                              sm.act + warp * row_list_bytes(N), K.rl2u, nb, mycol, ncols,
                              S.raw ? S.raw + rd.nbr_off : nbg + (size_t)N * P * cap_sub,
-                             (uint32_t)(i * P + q), (uint32_t)(N * P),
-                             S.raw ? cap_sub / 4 : list_notes(E.cap, cap_sub, P), cap_sub, &overflow);
+                             (uint32_t)(i * P + q), (uint32_t)(N * P), notes, cap_sub, &overflow);
       // the FP64 pair loop's notes overlie the screening vectors
       if (FP64 && P >= 4) __syncthreads();
     }

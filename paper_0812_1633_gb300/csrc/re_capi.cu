@@ -424,18 +424,38 @@ int upload_tables(re_ctx* c) {
   return RE_OK;
 }
 
-// Allocate device memory for the current ens/reps tables.
-// Whether a screened list build (see re_batched.cuh) of some launch shape would
-// find next to no room for its notes in the list array: sparse systems and
-// capacities given by the caller.  An array of their own then holds them.
-bool notes_need_room(const re_ctx* c) {
-  if (c->opt.path != RE_PATH_BATCHED) return false;
-  for (const EnsDev& e : c->ens)
-    for (int k = 0; k < 3; ++k)
-      if (e.N > re::kDirectBuild && re::list_notes(e.cap, e.capsub[k], 1 << k) < 4) return true;
-  return false;
+// Whether a screened list build (see re_batched.cuh) in shape k finds room for less
+// than half of the notes that a lane can make in the list array: four threads an
+// atom, sparse systems, capacities given by the caller.
+bool notes_short(const EnsDev& e, const LaunchCfg& k) {
+  const int P = k.atom_threads, idx = P == 1 ? 0 : (P == 2 ? 1 : 2);
+  if (P > 4 || e.N <= re::kDirectBuild) return false;
+  const int quads = (e.N + 127) / 128;  // of rows; a lane makes 4 / P notes of each
+  return 2 * re::list_notes(e.cap, e.capsub[idx], P) < std::min(e.capsub[idx] / 4, quads * (4 / P));
 }
 
+// An array of their own for the notes, while a launch shape in use is short of room
+// for them: 1372 atoms on eight CTAs of four threads an atom, skin 0.1, 15.1 us a
+// step instead of 16.4.  Such shapes are those of few replicas; the others do
+// without it.  Failing to get it changes the time only.  Given back only where no
+// cached graph can hold it (give_back: the graphs are dropped there).
+void fit_notes(re_ctx* c, bool give_back) {
+  bool need = false;
+  for (size_t e = 0; e < c->ens.size() && c->opt.path == RE_PATH_BATCHED; ++e) {
+    need |= notes_short(c->ens[e], c->cfg) || (c->use_fcfg && notes_short(c->ens[e], c->fcfg));
+    if (per_class(c)) need |= notes_short(c->ens[e], c->ecfg[e]);
+  }
+  if (need == (c->s.raw != nullptr)) return;
+  const std::string err = c->err;
+  if (!need) {
+    if (give_back) dfree(c, c->s.raw);
+  } else if (dalloc(c, &c->s.raw, (size_t)c->n_nbr) != RE_OK) {
+    cudaGetLastError();
+    c->err = err;
+  }
+}
+
+// Allocate device memory for the current ens/reps tables.
 int allocate(re_ctx* c) {
   const size_t A = (size_t)c->n_atoms, R = (size_t)c->n_rep, E = c->ens.size();
   StateDev& s = c->s;
@@ -445,7 +465,6 @@ int allocate(re_ctx* c) {
       (rc = dalloc(c, &s.fx, A)) || (rc = dalloc(c, &s.fy, A)) || (rc = dalloc(c, &s.fz, A)) ||
       (rc = dalloc(c, &s.rx, A)) || (rc = dalloc(c, &s.ry, A)) || (rc = dalloc(c, &s.rz, A)) ||
       (rc = dalloc(c, &s.ncnt, 8 * A)) || (rc = dalloc(c, &s.nbr, (size_t)c->n_nbr)) ||
-      (notes_need_room(c) && (rc = dalloc(c, &s.raw, (size_t)c->n_nbr))) ||
       (rc = dalloc(c, &s.T, R)) || (rc = dalloc(c, &s.U, 4 * R)) || (rc = dalloc(c, &s.vscale, R)) ||
       (rc = dalloc(c, &s.lam, R)) || (rc = dalloc(c, &s.fscale, R)) ||
       (rc = dalloc(c, &s.step, R)) || (rc = dalloc(c, &s.nreb, R)) ||
@@ -466,6 +485,7 @@ int allocate(re_ctx* c) {
     return rc;
   // what is read back together lies together, laid out like h_out: the energies
   // and the status words, the partners and the decisions
+  fit_notes(c, false);
   s.K = s.U + R;
   s.econs = s.U + 2 * R;
   s.status = reinterpret_cast<int32_t*>(s.U + 3 * R);
@@ -1041,6 +1061,7 @@ int re_group(re_ctx* const* ctxs, int n, re_ctx** out) {
     if (c->opt.path == RE_PATH_BATCHED) rcode = check_cfg(c, c->cfg);
     if (rcode == RE_OK && per_class(c)) rcode = check_class_cfgs(c);
     if (rcode == RE_OK) rcode = upload_tables(c);
+    if (rcode == RE_OK) fit_notes(c, true);
   }
   // copy member states
   for (int i = 0; i < n && rcode == RE_OK; ++i) {
@@ -1250,6 +1271,7 @@ int re_run_free(re_ctx* c, int n_att, int nx, int64_t* log_step, double* log_T,
     RE_CUDA(c, cudaMemsetAsync(c->d_log_T, 0, 8 * n, c->stream), "clear log");
   }
   c->use_fcfg = narrower;
+  fit_notes(c, false);
   int rc = launch_advance(c, c->d_budget_nx, nullptr, n_att * nx, 0, &fr);
   c->use_fcfg = false;
   if (rc) return rc;
@@ -1927,6 +1949,7 @@ int re_checkpoint_load(re_ctx* c, const void* buf, size_t bytes) {
     cudaGraphExecDestroy(c->rec_graph);
     c->rec_graph = nullptr;
   }
+  fit_notes(c, true);
   size_t off = sizeof h + sizeof(LaunchCfg) * c->ens.size();
   for (const CkptArray& a : ckpt_arrays(c)) {
     if (a.bytes)
@@ -2144,6 +2167,7 @@ int re_autotune(re_ctx* c, int steps) {
             if (check_cfg(c, k, sc) != RE_OK) continue;
             if (ls == 1 && list_elems_for(c, k, sc) == 0) continue;
             c->ecfg[e] = k;
+            fit_notes(c, false);
             const float ms = trial([&](const int32_t* b) { return launch_class(c, e, b, c->stream); });
             if (ms < cbest_ms) {
               cbest_ms = ms;
@@ -2187,6 +2211,7 @@ int re_autotune(re_ctx* c, int steps) {
         if (check_cfg(c, k) != RE_OK) continue;
         if (ls == 1 && list_elems_for(c, k) == 0) continue;
         c->cfg = k;
+        fit_notes(c, false);
         float ms = trial([&](const int32_t* b) { return launch_advance(c, b, nullptr, 1); });
         // the split launch must win clearly: its gain is within the noise of
         // a trial on the workloads measured so far
@@ -2207,6 +2232,7 @@ int re_autotune(re_ctx* c, int steps) {
     apply_cells_each(c);
   else
     apply_cells(c, best_m);
+  fit_notes(c, true);  // the cached graphs go below
   upload_tables(c);
   for (auto& b : bufs) {
     cudaMemcpyAsync(b.dev, b.save, b.bytes, cudaMemcpyDeviceToDevice, c->stream);

@@ -151,7 +151,7 @@ struct StateDev {
   uint32_t *rx, *ry, *rz;
   int32_t* ncnt;
   uint16_t* nbr;
-  uint16_t* raw;  // as nbr: notes of the list builds, where list_notes() finds no room (else null)
+  uint16_t* raw;  // as nbr: notes of the list builds, where nbr has little room for them (else null)
   double *T, *U, *K, *econs, *vscale;
   double *lam, *fscale;  // per replica: potential scale; pending force factor
   int64_t *step, *nreb;

@@ -1,7 +1,7 @@
 """Device memory of a batched context: the state, one set of neighbour lists and
 the fixed words, at the default capacity and at one that leaves no room in the
 lists' array (where the build's notes get an array of their own, and the lists
-are the same)."""
+are the same), also after the autotuner has gone through shapes that need one."""
 import numpy as np
 import pytest
 
@@ -54,3 +54,25 @@ def test_capacity_without_room_for_notes(cap):
         else:
             d = out[0] - out[1]
             assert np.abs(d - L * np.rint(d / L)).max() < 1e-3
+
+
+def test_shapes_with_and_without_the_array():
+    """The tuner goes through shapes with and without room for notes, and a
+    free-running launch may take another one between replays of a cached graph."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_0812_1633_gb300 as re
+    N, R = 1372, 12
+    L, temps = inputs.box_length(N), [0.9 + 0.1 * k for k in range(R)]
+    a = re.Context(N, L, 2.5, temps, 5, skin=0.3)
+    cfg = a.autotune(steps=5)
+    b = re.Context(N, L, 2.5, temps, 5, skin=0.3, cluster=cfg["cluster"], atom_threads=cfg["atom_threads"])
+    assert np.array_equal(a.get_state()[0], b.get_state()[0])
+    for ctx in (a, b):
+        ctx.run(4, graph=True)
+        ctx.run_free(2, 5)
+        ctx.run(4, graph=True)
+        assert np.isfinite(ctx.energies()[0]).all()
+    a.close()
+    b.close()
