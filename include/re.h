@@ -324,7 +324,11 @@ int re_config_wide(const re_ctx *c, int *wide_n, int *wide_cluster, int *wide_th
  * the lists' placement, global or shared memory, and each as one launch or
  * split, see re_opts.wide_launch) in launches of `steps` steps, as the caller
  * will make them, on a copy of the state and keeps the fastest; the state is
- * restored afterwards.  cell_div is varied only while no shape is admitted.
+ * restored afterwards.  Every replica makes `steps` steps in a trial: calls whose
+ * budgets differ between replicas run in another order and, where even budgets
+ * would put two CTAs on an SM, in another register build, so that the shape
+ * kept is the fastest for even budgets.  cell_div is varied only while no shape
+ * is admitted.
  * With per-ensemble launches (re_opts.group_launch) every ensemble's shape is
  * tuned on its own launch. */
 int re_autotune(re_ctx *c, int steps);

@@ -2051,8 +2051,9 @@ int re_autotune(re_ctx* c, int steps) {
   ApiRange range_("re_autotune");
   if (!c) return fail(nullptr, RE_EINVAL, "context is NULL");
   if (c->opt.path != RE_PATH_BATCHED) return RE_OK;
-  // launches of as many steps as the caller's, whose fixed parts (start, lists
-  // copied to shared memory, a split launch's ordering) count as they do in use
+  // launches of as many steps as the caller's, the same for every replica, whose
+  // fixed parts (start, lists copied to shared memory, a split launch's ordering)
+  // count as they do in use
   steps = std::max(steps, 1);
   const int n_warm = (40 + steps - 1) / steps, n_timed = std::max(2, (120 + steps - 1) / steps);
   int rc = status_check(c);

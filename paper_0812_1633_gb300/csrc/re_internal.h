@@ -90,9 +90,9 @@ inline void set_pair_constants(StepConst& k) {
   double best = 1.0;
   for (uint32_t i = 0; i < 256 && best > 1e-9; ++i) {
     const double c1 = 0.5 + ((i * i * 0x9E3779u + i * 0x3C6EF3u) & 0x7FFFFFu) * 0x1.0p-24;
-    const double c3 = k3 * c1, off = std::fabs((double)(float)c3 / c3 - 1.0);
-    if (off >= best) continue;
-    best = off;
+    const double c3 = k3 * c1, off = std::fabs((double)(float)c3 - c3);
+    if (off >= best * c3) continue;
+    best = off / c3;
     k.c1 = (float)c1;
     k.c3 = (float)c3;
   }

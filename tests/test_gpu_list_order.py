@@ -70,6 +70,7 @@ def check(ctx, N, L, R, prec):
         assert U[r] == pytest.approx(uo, rel=1e-10 if prec == "fp64" else 1e-6)
 
 
+@pytest.mark.parametrize("smem", [-1, 1])
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("N,P,cluster,order", [
     (256, 8, 2, "4"), (500, 4, 4, "4"), (864, 8, 8, "octants"),   # every atom tested
@@ -77,12 +78,12 @@ def check(ctx, N, L, R, prec):
     (1372, 4, 8, "4"), (1372, 2, 4, "2"),                         # last row partly filled
     (2048, 4, 8, "4"), (2048, 4, 8, "16"), (2048, 4, 8, "random"), (2048, 2, 4, "32"),
 ])
-def test_any_numbering(re, N, P, cluster, order, prec):
+def test_any_numbering(re, N, P, cluster, order, prec, smem):
     x, L = liquid(N, N)
     R = 2
     xs = np.concatenate([reorder(x, L, order, 1), reorder(x, L, order, 2)])
     ctx = re.Context(N, L, 2.5, [1.0, 1.3], 5, precision=prec, cluster=cluster, atom_threads=P,
-                     sort_interval=-1)
+                     sort_interval=-1, lists_smem=smem)
     ctx.set_state(xs)
     check(ctx, N, L, R, prec)
     ctx.advance(30)
