@@ -942,16 +942,16 @@ def run_diffusion(args):
 
 
 # DRAM bytes (read + write) per launch of the advance kernel, from one ncu
-# capture per workload and launch shape (profiles/md_batched_kernel_64x864.md),
+# capture per workload and launch shape (its summary is in profiles/),
 # valid only while the kernel's sources are the ones that were profiled.
 PROFILED_TRAFFIC = {
-    ("c1", (2, 2, 2), "mixed"): {"kernel_sha256_16": "a4ad8bc1e28300ab",
-                                 "bytes_per_launch": 13372416 + 114432,
+    ("c1", (2, 2, 2), "mixed"): {"kernel_sha256_16": "9b8dd646a6bec915",
+                                 "bytes_per_launch": 14288896 + 69376,
                                  # pipe use over the SMs' active cycles (ncu --set full)
-                                 "pipes": {"fma_pct": 20.37, "alu_pct": 42.45, "fp64_pct": 4.54,
-                                           "issue_active_pct": 54.64,
-                                           "smem_wavefronts": 18331402,
-                                           "smem_bank_conflicts": 7500934}},
+                                 "pipes": {"fma_pct": 19.94, "alu_pct": 40.73, "fp64_pct": 4.46,
+                                           "issue_active_pct": 53.41,
+                                           "smem_wavefronts": 18227323,
+                                           "smem_bank_conflicts": 7456171}},
 }
 
 

@@ -440,13 +440,13 @@ __device__ int build_list_cells(int i, PosFn pos_hi, int N, int nc, int m, const
 // so the least sum at a given r^2 is the one of equal components).  One
 // mma.m16n8k8 (f16 vectors, f32 sums; the other two of its eight products add
 // the limit, and put the last row's missing atoms beyond it) screens 16 atoms
-// against 8; one funnel shift per result collects its sign.  Of the candidates that pass (7 to 20 % more than the list at
-// L = 17 to 10) the exact test on the 32-bit positions keeps the list, so the
-// pair set does not depend on the screening.  No cells are built or sorted: a
-// warp goes through the rows (32 consecutive atoms) whose bounding box lies
-// within the list radius of its own atoms' box.  Atoms are renumbered in space
-// order from time to time, so both boxes are small; the order affects the time
-// only.
+// against 8; one funnel shift per result collects its sign.  Of the candidates that
+// pass (7 to 20 % more than the list at L = 17 to 10) the exact test on the 32-bit
+// positions keeps the list, so the pair set does not depend on the screening.  No
+// cells are built or sorted: a warp goes through the rows (32 consecutive atoms)
+// whose bounding box lies within the list radius of its own atoms' box.  Atoms are
+// renumbered in space order from time to time, so both boxes are small; the order
+// affects the time only.
 //
 // A lane's hits come unevenly from mask to mask, but in all the lanes of a warp
 // have nearly the same number.  So the masks are only noted, and the loop over
